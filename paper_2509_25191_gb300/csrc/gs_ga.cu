@@ -643,20 +643,37 @@ __global__ void __launch_bounds__(GA_SEL_THREADS) k_ga_inc_sort(const int32_t *_
 }
 
 // ---------------------------------------------------------------------------
-// Weights (Eq. 3) and median order statistics (Eq. 4).
-// scratch words: [0] max bits, [1] radix prefix, [2] rank, [8..8+2048) radix
-// histogram, [8+2048..) per-bin weight table (floats).
+// Weights (Eq. 3) and median order statistics (Eq. 4), in three passes over the
+// distances: (a) the maximum and a histogram of the top 10 key bits (a key is a
+// distance's float bits); (b) the bin counts and the next 11 bits of the keys
+// that share the lower median's top bits; (c) the weights and the last 11 bits.
+// The last block of each pass to finish picks the pass's digit of the lower
+// median (and in (b) forms the table of weights), so no launch lies between the
+// passes. The upper median is the next key: in the same final histogram, or the
+// smallest key above its range, which (c) keeps as a minimum.
+// Bound: 4 B read per pass and 4 B written (HBM for the first pass, mostly L2
+// after it where the distances fit). 21.3M distances: 92 us, against 285 us for
+// nine passes with six one-warp digit picks between them; counters in one copy per block
+// alone took 46 us for the bin counts, since most distances fall into the first
+// few bins and the lanes of a warp then queue for one address. Here neighbouring
+// lanes count in different copies (up to 32) of the counters.
+// scratch words: [0] max bits, [1] prefix of the lower median's key, [2] its rank
+// among the keys with that prefix, [3..5] blocks done per pass, [6] smallest key
+// above the prefix's range (complemented), [8..8+2048) digit histogram,
+// [8+2048..) per-bin weight table (floats).
 // ---------------------------------------------------------------------------
 constexpr int GA_W_HIST = 8;
 constexpr int GA_W_TABLE = 8 + GA_RADIX_BINS;
+constexpr int GA_W_THREADS = 512;
+constexpr int GA_W_B0 = 10, GA_W_B1 = 11, GA_W_B2 = 11;   // bits of the key's digits from the top
+constexpr int GA_W_COPY_WORDS = 16384;       // shared words for the copies of a pass's first counters
+static_assert(GA_W_B0 + GA_W_B1 + GA_W_B2 == 32 && (1 << GA_W_B1) <= GA_RADIX_BINS, "key digits");
 
-__global__ void __launch_bounds__(256) k_ga_max(const float *__restrict__ e, long long n, uint32_t *scratch) {
-    uint32_t mx = 0;
-    for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += (long long)gridDim.x * 256)
-        mx = max(mx, __float_as_uint(e[k]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&scratch[0], mx);
+// copies of nb counters (a power of two, at most 32) that fit the shared words
+__host__ __device__ inline int ga_copies(int nb) {
+    int c = 32;
+    while (c > 1 && c * nb > GA_W_COPY_WORDS) c >>= 1;
+    return c;
 }
 
 __device__ __forceinline__ int ga_bin(float e, float inv, int nb, bool any) {
@@ -664,27 +681,123 @@ __device__ __forceinline__ int ga_bin(float e, float inv, int nb, bool any) {
     return max(0, min(nb - 1, (int)floorf(__fmul_rn(e, inv))));
 }
 
-__global__ void __launch_bounds__(256) k_ga_hist(const float *__restrict__ e, long long n, int nb,
-                                                 const uint32_t *__restrict__ scratch, uint32_t *counts) {
-    extern __shared__ uint32_t s_h[];
-    for (int b = threadIdx.x; b < nb; b += 256) s_h[b] = 0;
-    __syncthreads();
-    const float emax = __uint_as_float(scratch[0]);
-    const bool any = emax > 0.f;
-    const float inv = any ? __fdiv_rn((float)nb, emax) : 0.f;
-    for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += (long long)gridDim.x * 256)
-        atomicAdd(&s_h[ga_bin(e[k], inv, nb, any)], 1u);
-    __syncthreads();
-    for (int b = threadIdx.x; b < nb; b += 256)
-        if (s_h[b]) atomicAdd(&counts[b], s_h[b]);
+// f(value, index) over all n distances with the whole grid: 16-byte loads of
+// four neighbours where the array is 16-byte aligned (two in flight per thread),
+// the tail (or a misaligned array) one by one. f4(values, first index) takes a
+// whole group.
+template <typename F4, typename F1>
+__device__ __forceinline__ void ga_each(const float *__restrict__ e, long long n, F4 &&f4, F1 &&f1) {
+    const long long stride = (long long)gridDim.x * GA_W_THREADS, t = (long long)blockIdx.x * GA_W_THREADS + threadIdx.x;
+    const long long n4 = ((uintptr_t)e & 15u) == 0 ? n >> 2 : 0;
+    const float4 *e4 = reinterpret_cast<const float4 *>(e);
+    long long k = t;
+    for (; k + stride < n4; k += 2 * stride) {
+        const float4 a = e4[k], b = e4[k + stride];
+        f4(a, 4 * k);
+        f4(b, 4 * (k + stride));
+    }
+    if (k < n4) f4(e4[k], 4 * k);
+    for (k = 4 * n4 + t; k < n; k += stride) f1(e[k], k);
 }
 
-__global__ void __launch_bounds__(256) k_ga_table(const uint32_t *__restrict__ counts, int nb, long long n,
-                                                  double alpha, uint32_t *scratch) {
+// true in every thread of the last block to get here (its other blocks' global
+// writes are then visible to it)
+__device__ __forceinline__ bool ga_last_block(uint32_t *done) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
+}
+
+// The digit of the histogram (2^bits bins, bits 10 or 11) that holds the rank:
+// scratch[1] |= digit << shift, scratch[2] becomes the rank within the digit, the
+// histogram is cleared. Whole block; returns the digit, and in *count the number
+// of keys in it.
+template <int BITS>
+__device__ __forceinline__ uint32_t ga_pick(uint32_t *scratch, uint32_t rank, int shift, uint32_t *count) {
+    constexpr int PER = (1 << BITS) / GA_W_THREADS;
+    __shared__ uint32_t s_part[GA_W_THREADS / 32], s_digit, s_count;
+    uint32_t *h = scratch + GA_W_HIST;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t c[PER], local = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        c[k] = __ldcg(h + threadIdx.x * PER + k);
+        local += c[k];
+    }
+    uint32_t incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) s_part[wid] = incl;
+    __syncthreads();
+    for (int w = 0; w < wid; ++w) incl += s_part[w];
+    uint32_t at = incl - local;
+    if (rank >= at && rank < incl) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            if (rank >= at && rank - at < c[k]) {
+                s_digit = (uint32_t)(threadIdx.x * PER + k);
+                s_count = c[k];
+                scratch[1] |= s_digit << shift;
+                scratch[2] = rank - at;
+            }
+            at += c[k];
+        }
+    }
+    __syncthreads();
+    if (count) *count = s_count;
+    return s_digit;
+}
+
+template <int BITS>
+__device__ __forceinline__ void ga_clear_hist(uint32_t *scratch) {
+    for (int b = threadIdx.x; b < (1 << BITS); b += GA_W_THREADS) scratch[GA_W_HIST + b] = 0u;
+}
+
+__global__ void __launch_bounds__(GA_W_THREADS) k_ga_w_max(const float *__restrict__ e, long long n, int copies,
+                                                           uint32_t rank, uint32_t *scratch) {
+    extern __shared__ uint32_t s_h[];
+    constexpr int NB = 1 << GA_W_B0, SH = 32 - GA_W_B0;
+    for (int b = threadIdx.x; b < NB * copies; b += GA_W_THREADS) s_h[b] = 0u;
+    __syncthreads();
+    uint32_t mx = 0u;
+    uint32_t *mine = s_h + (threadIdx.x & (copies - 1));
+    auto one = [&](float v, long long) {
+        const uint32_t key = __float_as_uint(v);
+        mx = max(mx, key);
+        atomicAdd(mine + (key >> SH) * copies, 1u);
+    };
+    ga_each(e, n, [&](const float4 &v, long long k) { one(v.x, k); one(v.y, k); one(v.z, k); one(v.w, k); }, one);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&scratch[0], mx);
+    __syncthreads();
+    for (int b = threadIdx.x; b < NB; b += GA_W_THREADS) {
+        uint32_t c = 0u;
+        for (int k = 0; k < copies; ++k) c += s_h[b * copies + ((k + threadIdx.x) & (copies - 1))];
+        if (c) atomicAdd(&scratch[GA_W_HIST + b], c);
+    }
+    if (!ga_last_block(scratch + 3)) return;
+    ga_pick<GA_W_B0>(scratch, rank, SH, nullptr);
+    ga_clear_hist<GA_W_B0>(scratch);
+}
+
+// The table of weights from the bin counts (one block): w_b = (n c_b / sum c^2)^alpha
+__device__ __forceinline__ void ga_table(const uint32_t *counts, int nb, long long n, double alpha, uint32_t *scratch) {
     __shared__ double s_part[256];
     double s2 = 0.0;
-    for (int b = threadIdx.x; b < nb; b += 256) s2 += (double)counts[b] * (double)counts[b];
-    s_part[threadIdx.x] = s2;
+    if (threadIdx.x < 256) {
+        for (int b = threadIdx.x; b < nb; b += 256) {
+            const double c = (double)__ldcg(counts + b);
+            s2 += c * c;
+        }
+        s_part[threadIdx.x] = s2;
+    }
     __syncthreads();
     for (int o = 128; o > 0; o >>= 1) {
         if (threadIdx.x < o) s_part[threadIdx.x] += s_part[threadIdx.x + o];
@@ -692,75 +805,98 @@ __global__ void __launch_bounds__(256) k_ga_table(const uint32_t *__restrict__ c
     }
     const double S2 = s_part[0];
     float *table = reinterpret_cast<float *>(scratch + GA_W_TABLE);
-    for (int b = threadIdx.x; b < nb; b += 256)
-        table[b] = counts[b] ? (float)pow((double)n * (double)counts[b] / S2, alpha) : 0.f;
+    for (int b = threadIdx.x; b < nb; b += GA_W_THREADS) {
+        const uint32_t c = __ldcg(counts + b);
+        table[b] = c ? (float)pow((double)n * (double)c / S2, alpha) : 0.f;
+    }
 }
 
-__global__ void __launch_bounds__(256) k_ga_gather(const float *__restrict__ e, long long n, int nb,
-                                                   const uint32_t *__restrict__ scratch, float *w) {
+__global__ void __launch_bounds__(GA_W_THREADS) k_ga_w_count(const float *__restrict__ e, long long n, int nb,
+                                                             int copies, double alpha, uint32_t *scratch,
+                                                             uint32_t *counts) {
+    extern __shared__ uint32_t s_h[];   // the bin counters' copies, then the digit histogram
+    constexpr int SH = 32 - GA_W_B0 - GA_W_B1, DIG = 1 << GA_W_B1;
+    uint32_t *s_d = s_h + nb * copies;
+    for (int b = threadIdx.x; b < nb * copies + DIG; b += GA_W_THREADS) s_h[b] = 0u;
+    __syncthreads();
     const float emax = __uint_as_float(scratch[0]);
     const bool any = emax > 0.f;
     const float inv = any ? __fdiv_rn((float)nb, emax) : 0.f;
-    const float *table = reinterpret_cast<const float *>(scratch + GA_W_TABLE);
-    for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += (long long)gridDim.x * 256)
-        w[k] = table[ga_bin(e[k], inv, nb, any)];
+    const uint32_t top = scratch[1] >> (32 - GA_W_B0);
+    uint32_t *mine = s_h + (threadIdx.x & (copies - 1));
+    auto one = [&](float v, long long) {
+        atomicAdd(mine + ga_bin(v, inv, nb, any) * copies, 1u);
+        const uint32_t key = __float_as_uint(v);
+        if (key >> (32 - GA_W_B0) == top) atomicAdd(s_d + ((key >> SH) & (DIG - 1)), 1u);
+    };
+    ga_each(e, n, [&](const float4 &v, long long k) { one(v.x, k); one(v.y, k); one(v.z, k); one(v.w, k); }, one);
+    __syncthreads();
+    for (int b = threadIdx.x; b < nb; b += GA_W_THREADS) {
+        uint32_t c = 0u;
+        for (int k = 0; k < copies; ++k) c += s_h[b * copies + ((k + threadIdx.x) & (copies - 1))];
+        if (c) atomicAdd(&counts[b], c);
+    }
+    for (int b = threadIdx.x; b < DIG; b += GA_W_THREADS)
+        if (s_d[b]) atomicAdd(&scratch[GA_W_HIST + b], s_d[b]);
+    if (!ga_last_block(scratch + 4)) return;
+    ga_table(counts, nb, n, alpha, scratch);
+    ga_pick<GA_W_B1>(scratch, scratch[2], SH, nullptr);
+    ga_clear_hist<GA_W_B1>(scratch);
 }
 
-// Radix select of the rank-th smallest key (float bits of e >= 0): three
-// digit passes of 11, 11 and 10 bits from the top.
-__global__ void __launch_bounds__(256) k_ga_radix_hist(const float *__restrict__ e, long long n, int shift, int bits,
-                                                       uint32_t pmask, uint32_t *scratch) {
-    __shared__ uint32_t s_h[GA_RADIX_BINS];
-    for (int b = threadIdx.x; b < GA_RADIX_BINS; b += 256) s_h[b] = 0;
+__global__ void __launch_bounds__(GA_W_THREADS) k_ga_w_gather(const float *__restrict__ e, long long n, int nb,
+                                                              uint32_t *scratch, float *__restrict__ w, float *stats) {
+    extern __shared__ uint32_t s_h[];   // the digit histogram, then the table of weights
+    constexpr int DIG = 1 << GA_W_B2;
+    float *s_table = reinterpret_cast<float *>(s_h + DIG);
+    for (int b = threadIdx.x; b < DIG; b += GA_W_THREADS) s_h[b] = 0u;
+    for (int b = threadIdx.x; b < nb; b += GA_W_THREADS)
+        s_table[b] = reinterpret_cast<const float *>(scratch + GA_W_TABLE)[b];
     __syncthreads();
-    const uint32_t prefix = scratch[1];
-    const uint32_t dmask = (1u << bits) - 1u;
-    for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += (long long)gridDim.x * 256) {
-        const uint32_t key = __float_as_uint(e[k]);
-        if ((key & pmask) == prefix) atomicAdd(&s_h[(key >> shift) & dmask], 1u);
-    }
+    const float emax = __uint_as_float(scratch[0]);
+    const bool any = emax > 0.f;
+    const float inv = any ? __fdiv_rn((float)nb, emax) : 0.f;
+    const uint32_t top = scratch[1] >> GA_W_B2;
+    uint32_t above = 0u;   // the largest complement of a key above the prefix's range
+    auto one = [&](float v) {
+        const uint32_t key = __float_as_uint(v), t = key >> GA_W_B2;
+        if (t == top) atomicAdd(s_h + (key & (DIG - 1)), 1u);
+        else if (t > top) above = max(above, ~key);
+        return s_table[ga_bin(v, inv, nb, any)];
+    };
+    const bool w4 = ((uintptr_t)w & 15u) == 0;
+    ga_each(e, n,
+            [&](const float4 &v, long long k) {
+                const float4 r = make_float4(one(v.x), one(v.y), one(v.z), one(v.w));
+                if (w4) {
+                    *reinterpret_cast<float4 *>(w + k) = r;
+                } else {
+                    w[k] = r.x; w[k + 1] = r.y; w[k + 2] = r.z; w[k + 3] = r.w;
+                }
+            },
+            [&](float v, long long k) { w[k] = one(v); });
+    above = __reduce_max_sync(0xffffffffu, above);
+    if ((threadIdx.x & 31) == 0 && above) atomicMax(&scratch[6], above);
     __syncthreads();
-    for (int b = threadIdx.x; b < GA_RADIX_BINS; b += 256)
+    for (int b = threadIdx.x; b < DIG; b += GA_W_THREADS)
         if (s_h[b]) atomicAdd(&scratch[GA_W_HIST + b], s_h[b]);
-}
-
-__global__ void k_ga_radix_init(uint32_t *scratch, uint32_t rank) {
-    scratch[1] = 0u;
-    scratch[2] = rank;
-}
-
-// One warp: find the digit holding the rank, extend the prefix, subtract the
-// keys below it from the rank, clear the histogram for the next pass.
-__global__ void k_ga_radix_pick(int shift, int bits, uint32_t *scratch, float *stats_out) {
-    const int lane = threadIdx.x;
-    const int nbins = 1 << bits, per = nbins / 32;
-    uint32_t *h = scratch + GA_W_HIST;
-    uint32_t rank = scratch[2];
-    uint32_t local = 0;
-    for (int k = 0; k < per; ++k) local += h[lane * per + k];
-    // inclusive scan across lanes
-    uint32_t incl = local;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    const uint32_t excl = incl - local;
-    const bool mine = rank >= excl && rank < incl;
-    if (mine) {
-        uint32_t r = rank - excl;
-        int d = lane * per;
-        while (r >= h[d]) {
-            r -= h[d];
-            ++d;
+    if (!ga_last_block(scratch + 5)) return;
+    uint32_t in_digit;
+    const uint32_t digit = ga_pick<GA_W_B2>(scratch, scratch[2], 0, &in_digit);
+    if (threadIdx.x == 0) {
+        const uint32_t lo = scratch[1];
+        uint32_t hi = lo;
+        if ((n & 1) == 0 && scratch[2] + 1u >= in_digit) {
+            // the next key: the next bin of this histogram, or the smallest above
+            uint32_t d = digit + 1;
+            while (d < DIG && __ldcg(scratch + GA_W_HIST + d) == 0u) ++d;
+            hi = d < DIG ? (top << GA_W_B2) | d : ~__ldcg(scratch + 6);
         }
-        const uint32_t prefix = scratch[1] | ((uint32_t)d << shift);
-        scratch[1] = prefix;
-        scratch[2] = r;
-        if (stats_out) *stats_out = __uint_as_float(prefix);
+        stats[0] = emax;
+        stats[1] = __uint_as_float(lo);
+        stats[2] = __uint_as_float(hi);
+        stats[3] = 0.f;
     }
-    __syncwarp();
-    for (int k = lane; k < nbins; k += 32) h[k] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -841,33 +977,28 @@ int launch_ga_step(const gs_ga_state &s, const gs_ga_problem &P, float *pair_sum
 
 int launch_ga_weights(const float *e, long long n, int nb, double alpha, uint32_t *counts, float *w, float *stats,
                       uint32_t *scratch, cudaStream_t st) {
-    const size_t words = (size_t)GA_W_TABLE + (size_t)nb;
-    if (cudaMemsetAsync(scratch, 0, words * 4, st) != cudaSuccess) return GS_ERR_CUDA;
-    if (cudaMemsetAsync(stats, 0, 4 * sizeof(float), st) != cudaSuccess) return GS_ERR_CUDA;
+    // (the table is written before it is read)
+    if (cudaMemsetAsync(scratch, 0, (size_t)GA_W_TABLE * 4, st) != cudaSuccess) return GS_ERR_CUDA;
     if (cudaMemsetAsync(counts, 0, (size_t)nb * 4, st) != cudaSuccess) return GS_ERR_CUDA;
-    if (n == 0) return GS_OK;
-    const int grid = 4 * num_sms();
-    k_ga_max<<<grid, 256, 0, st>>>(e, n, scratch);
-    const size_t smem = (size_t)nb * 4;
-    if (smem > 48 * 1024)
-        if (cudaFuncSetAttribute(k_ga_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return GS_ERR_CUDA;
-    k_ga_hist<<<2 * num_sms(), 256, smem, st>>>(e, n, nb, scratch, counts);
-    k_ga_table<<<1, 256, 0, st>>>(counts, nb, n, alpha, scratch);
-    k_ga_gather<<<grid, 256, 0, st>>>(e, n, nb, scratch, w);
-    if (cudaMemcpyAsync(stats, scratch, 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return GS_ERR_CUDA;
-    // median order statistics: ranks (n-1)/2 and n/2
-    const long long ranks[2] = {(n - 1) / 2, n / 2};
-    const int shifts[3] = {21, 10, 0}, bits[3] = {11, 11, 10};
-    for (int r = 0; r < 2; ++r) {
-        k_ga_radix_init<<<1, 1, 0, st>>>(scratch, (uint32_t)ranks[r]);
-        uint32_t pmask = 0;
-        for (int p = 0; p < 3; ++p) {
-            k_ga_radix_hist<<<grid, 256, 0, st>>>(e, n, shifts[p], bits[p], pmask, scratch);
-            k_ga_radix_pick<<<1, 32, 0, st>>>(shifts[p], bits[p], scratch, p == 2 ? stats + 1 + r : nullptr);
-            pmask |= ((1u << bits[p]) - 1u) << shifts[p];
-        }
-    }
+    if (n == 0) return cudaMemsetAsync(stats, 0, 4 * sizeof(float), st) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
+    // eight distances per thread or more, at most two blocks per SM (by the
+    // counters' copies in shared memory)
+    const long long want = (n + 8LL * GA_W_THREADS - 1) / (8LL * GA_W_THREADS);
+    const int grid = (int)(want < 2LL * num_sms() ? want : 2LL * num_sms());
+    const int c0 = ga_copies(1 << GA_W_B0), c1 = ga_copies(nb);
+    const size_t m0 = 4ull * c0 << GA_W_B0, m1 = 4ull * ((size_t)c1 * nb + (1 << GA_W_B1)),
+                 m2 = 4ull * ((1 << GA_W_B2) + (size_t)nb);
+    // (the largest each kernel is ever launched with: the same setting from every call)
+    const int most = 4 * (GA_W_COPY_WORDS + GA_RADIX_BINS);
+    static_assert(GS_GA_MAX_BINS <= GA_W_COPY_WORDS, "one copy of the bin counters fits");
+    if (cudaFuncSetAttribute(k_ga_w_max, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+        cudaFuncSetAttribute(k_ga_w_count, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+        cudaFuncSetAttribute(k_ga_w_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
+        return GS_ERR_CUDA;
+    // the lower median's rank; the upper one is the next key if n is even
+    k_ga_w_max<<<grid, GA_W_THREADS, m0, st>>>(e, n, c0, (uint32_t)((n - 1) / 2), scratch);
+    k_ga_w_count<<<grid, GA_W_THREADS, m1, st>>>(e, n, nb, c1, alpha, scratch, counts);
+    k_ga_w_gather<<<grid, GA_W_THREADS, m2, st>>>(e, n, nb, scratch, w, stats);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 

@@ -311,3 +311,30 @@ def test_unfused_iteration_converges_like_the_fused_one():
         G.check()
         out.append(_rel_rot_err(tv.astype(np.float64), vm1.detach().cpu().numpy().astype(np.float64), pairs))
     assert out[0] < 0.3 * e0 and out[1] < 0.3 * e0, (e0, out)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 4096, 4097, 70001])
+@pytest.mark.parametrize("n_bins", [1, 100, 700, 16384])
+@pytest.mark.parametrize("kind", ["spread", "gap", "misaligned"])
+def test_weights_three_passes_at_their_edges(n, n_bins, kind):
+    """Sizes around a vector, a block and a grid; one to all copies of the bin
+    counters; an even count whose upper median lies in another key range than
+    the lower one; an array that does not start on 16 bytes."""
+    rng = np.random.default_rng(n + n_bins)
+    e = np.abs(rng.normal(0.0, 6.0, n)).astype(np.float32)
+    if kind == "gap" and n > 1:
+        e[: n // 2] = 1.0 + np.arange(n // 2, dtype=np.float32) * np.float32(2.0 ** -20)
+        e[n // 2:] = 300.0 + np.arange(n - n // 2, dtype=np.float32)
+        rng.shuffle(e)
+    d = torch.zeros(n + 1, device="cuda")
+    at = 1 if kind == "misaligned" else 0
+    d[at:at + n] = torch.as_tensor(e)
+    w, counts, stats = ga.pdf_weights(d[at:at + n], n_bins, 0.5)
+    torch.cuda.synchronize()
+    w_or, c_or = OG.pdf_weights(e, n_bins, 0.5)
+    assert (counts.cpu().numpy().astype(np.int64) == c_or).all()
+    # w is formed in double per bin and rounded once: half a unit in the last place of float32
+    assert np.allclose(w.cpu().numpy(), w_or, rtol=2.0 ** -23, atol=0)
+    lo, hi, _ = OG.median_order_stats(e)
+    st = stats.cpu().numpy()
+    assert st[0] == e.max() and st[1] == np.float32(lo) and st[2] == np.float32(hi) and st[3] == 0
