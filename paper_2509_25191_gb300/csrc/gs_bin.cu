@@ -21,7 +21,7 @@
 //   k_split_large  tiles far above the sort's work per block: partitioned
 //                  by depth into runs of bins, listed for the sort
 //   k_sort_tiles   persistent, one queue: the runs, then the other tiles
-//                  largest first; radix sort on chip
+//                  largest first; distribution sort on chip
 #include "gs_common.cuh"
 
 namespace gsk {
@@ -313,67 +313,61 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin_scatter(const Launch L, con
 }
 
 // ---------------------------------------------------------------------------
-// per-tile sort: stable block-wide LSD radix sort (8-bit digits) of a 16-bit
-// monotone compression of the depth bits, carrying the slot, then a fix-up
-// that orders each run of equal compressed keys by (depth bits, slot). The
-// result is the unique (depth, slot) order. Tiles longer than SORT_CAP
-// are sorted in chunks and merged (merge path) through keys_tmp.
+// per-tile sort on chip: a distribution sort whose buckets follow the tile's own
+// depths. The keys (held in registers) are counted into 1,024 bins of the top
+// bits of (depth bits - minimum); a bin's keys then get as many buckets as it
+// has keys, by the bits below, so that n keys meet n buckets whatever the
+// depths' density (clusters). Buckets are counted with shared-memory atomics,
+// whose results place the keys; the few keys of one bucket are ordered by
+// (depth bits, slot) by counting the smaller ones. The result is the unique
+// (depth, slot) order. Tiles longer than SORT_CAP are sorted in chunks and
+// merged (merge path) through keys_tmp.
+// Bound by instruction issue (0.6-0.7 per scheduler and cycle) and barriers:
+// eight keys per thread and three blocks of 512 threads per SM. A two-pass radix
+// sort (eight ballots per digit) took 12.2 warp instructions per instance and
+// 48 us on the 1M view's 2.38M instances at 32x32 tiles, 310 us on the 16-view
+// orbit; this one 9.5 and 35 us, 253 us. (256 threads x 4 blocks: the 8-view 6M
+// step 11.25 ms against 10.84; 8,192 keys on chip with 512 x 2 or 1024 x 2
+// threads: 11.35, 11.08.)
 // ---------------------------------------------------------------------------
-constexpr int SORT_THREADS = 256;
+constexpr int SORT_THREADS = 512;
 constexpr int SORT_WARPS = SORT_THREADS / 32;
-constexpr int SORT_CAP = 4096;      // ~74 KB of shared memory: 3 blocks per SM (228 KB with the per-block reserve)
-constexpr int SORT_SEG_MIN = 128;   // at least this many keys per active warp
+constexpr int SORT_CAP = 4096;
+constexpr int SORT_PER = SORT_CAP / SORT_THREADS;   // keys of a thread
+constexpr int SORT_BIN_BITS = 10, SORT_BINS = 1 << SORT_BIN_BITS;
+constexpr int SORT_BIN_PER = SORT_BINS / SORT_THREADS;   // bins of a thread in the scan
+static_assert(SORT_THREADS % 256 == 0 && SORT_PER % 4 == 0 && SORT_BIN_PER >= 1, "whole vectors per thread in the scans");
+
+constexpr int FIX_RUN = 32;   // most keys of a bucket that are ordered by counting
 
 struct SortSmem {
-    unsigned int key[2][SORT_CAP];
-    unsigned int val[2][SORT_CAP];
-    unsigned int hist[256][SORT_WARPS + 1];   // [digit][warp] counts, then running offsets (odd pitch)
-    unsigned int part[SORT_WARPS];   // per-warp partial sums of the histogram scan
-    unsigned int kmin, kmax;
+    unsigned int key[SORT_CAP], val[SORT_CAP];
+    uint4 bucket4[SORT_CAP / 4 + 1];       // per bucket: count, then first position; [n] = n
+    unsigned int bin[SORT_BINS + 1];       // per bin: count, then first bucket
+    unsigned int part[SORT_WARPS];         // per-warp partial sums of the scans
+    unsigned int kmin, kmax, nlong;
     int item;
-    unsigned int moff[257];          // large tiles: bin offsets within the tile
+    unsigned int lrun[2 * (SORT_CAP / (FIX_RUN + 1))];   // buckets of more than FIX_RUN keys: start, length
+    unsigned int moff[257];                // large tiles: bin offsets within the tile
 };
-// (the per-bin counts and cursors of a large tile's partition pass live in
-// hist, unused until the segments are sorted)
 
-// exclusive scan of the (digit, warp)-ordered counts hist[d][w], w < nwa:
-// thread d owns digit d (SORT_THREADS == 256 digits), sums its row, the block
-// scans the 256 row sums, and each row is rewritten as running offsets
-static_assert(SORT_THREADS == 256, "one thread per 8-bit digit");
-__device__ __forceinline__ void scan_hist(SortSmem &S, int nwa) {
-    const int d = threadIdx.x;
-    unsigned int sum = 0;
-    for (int w = 0; w < nwa; ++w) sum += S.hist[d][w];
+// exclusive sum over the block of one value per thread (two barriers)
+__device__ __forceinline__ unsigned int block_excl_sum(SortSmem &S, unsigned int x) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned int incl = sum;
+    unsigned int incl = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
+        const unsigned int t = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += t;
     }
     if (lane == 31) S.part[wid] = incl;
     __syncthreads();
-    if (wid == 0) {
-        unsigned int w = lane < SORT_WARPS ? S.part[lane] : 0, wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned int t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
-        }
-        if (lane < SORT_WARPS) S.part[lane] = wi - w;
-    }
-    __syncthreads();
-    unsigned int run = S.part[wid] + incl - sum;
-    for (int w = 0; w < nwa; ++w) {
-        const unsigned int c = S.hist[d][w];
-        S.hist[d][w] = run;
-        run += c;
-    }
-    __syncthreads();
+    // every warp sums the warps before it (16 partial sums, one per lane)
+    unsigned int before = lane < wid ? S.part[lane & (SORT_WARPS - 1)] : 0u;
+    before = __reduce_add_sync(0xffffffffu, before);
+    __syncthreads();   // part may be written again
+    return before + incl - x;
 }
-
-constexpr int FIX_RUN = 32;   // longest run of equal compressed keys one thread orders alone
-static_assert(2 * (SORT_CAP / (FIX_RUN + 1)) + 1 <= 256 * (SORT_WARPS + 1), "the long-run list fits the histogram");
 
 // Order key[0..L), val[0..L) (shared memory) by (key, val) with the whole
 // block: a sorting network of ascending compare-exchanges over the next power
@@ -411,20 +405,31 @@ __device__ void block_sort_run(unsigned int *key, unsigned int *val, int L) {
 
 // sort src[st .. st+n) (n <= SORT_CAP) by (depth, slot) into keys[st ..]
 // (src may be keys itself)
-__device__ void radix_sort_tile(SortSmem &S, const unsigned long long *src, unsigned long long *keys,
-                                unsigned int *__restrict__ ids, int st, int n, bool write_ids) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) { S.kmin = 0xffffffffu; S.kmax = 0u; }
+__device__ __forceinline__ void sort_on_chip(SortSmem &S, const unsigned long long *src, unsigned long long *keys,
+                             unsigned int *__restrict__ ids, int st, int n, bool write_ids) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    unsigned int *bucket = reinterpret_cast<unsigned int *>(S.bucket4);
+    if (tid == 0) {
+        S.kmin = 0xffffffffu;
+        S.kmax = 0u;
+        S.nlong = 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < SORT_BIN_PER; ++j) S.bin[tid + j * SORT_THREADS] = 0u;
     __syncthreads();
+    unsigned int d[SORT_PER], v[SORT_PER], at[SORT_PER];
     unsigned int lmin = 0xffffffffu, lmax = 0u;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += SORT_THREADS) {
-        const unsigned long long k = src[st + i];
-        const unsigned int d = (unsigned int)(k >> 32);
-        S.key[0][i] = d;
-        S.val[0][i] = (unsigned int)(k & 0xffffffffu);
-        lmin = min(lmin, d);
-        lmax = max(lmax, d);
+#pragma unroll
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        const int i = tid + j * SORT_THREADS;
+        if (i < n) {
+            const unsigned long long k = src[st + i];
+            d[j] = (unsigned int)(k >> 32);
+            v[j] = (unsigned int)(k & 0xffffffffu);
+            lmin = min(lmin, d[j]);
+            lmax = max(lmax, d[j]);
+        }
     }
     lmin = __reduce_min_sync(0xffffffffu, lmin);
     lmax = __reduce_max_sync(0xffffffffu, lmax);
@@ -433,98 +438,129 @@ __device__ void radix_sort_tile(SortSmem &S, const unsigned long long *src, unsi
         atomicMax(&S.kmax, lmax);
     }
     __syncthreads();
-    // Radix-sort a 16-bit monotone compression of the depth bits,
-    // (bits - kmin) >> shift, then order each run of equal compressed keys by
-    // the full (depth bits, slot): the same total order in at most 2 passes.
-    const unsigned int kmin = S.kmin, range = S.kmax - S.kmin;
+    const unsigned int kmin = S.kmin, range = S.kmax - kmin;
     const int nbits = range ? 32 - __clz(range) : 0;
-    const int shift = nbits > 16 ? nbits - 16 : 0;
-    const int passes = (min(nbits, 16) + 7) / 8;
-    const int nwa = max(1, min(SORT_WARPS, (n + SORT_SEG_MIN - 1) / SORT_SEG_MIN));
-    const int seg = ((n + nwa - 1) / nwa + 31) & ~31;
-    const int s0 = wid * seg, s1 = min(n, s0 + seg);
-    const unsigned int lt_mask = (1u << lane) - 1u;
-    int cur = 0;
-    for (int pass = 0; pass < passes; ++pass) {
-        const int dshift = shift + 8 * pass;
-        for (int w = 0; w < nwa; ++w) S.hist[threadIdx.x][w] = 0;
-        __syncthreads();
-        if (wid < nwa) {
-            // counts only: order does not matter, plain shared atomics
-            for (int i = s0 + lane; i < s1; i += 32)
-                atomicAdd(&S.hist[((S.key[cur][i] - kmin) >> dshift) & 255u][wid], 1u);
-        }
-        __syncthreads();
-        scan_hist(S, nwa);
-        if (wid < nwa) {
-            for (int b = s0; b < s1; b += 32) {
-                const int i = b + lane;
-                const bool act = i < s1;
-                const unsigned int key = act ? S.key[cur][i] : 0u;
-                const unsigned int d = ((key - kmin) >> dshift) & 255u;
-                // lanes holding the same digit, from one ballot per digit bit
-                unsigned int peers = __ballot_sync(0xffffffffu, act);
+    const int sh = max(0, nbits - SORT_BIN_BITS);
 #pragma unroll
-                for (int bit = 0; bit < 8; ++bit) {
-                    const unsigned int ones = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
-                    peers &= ((d >> bit) & 1u) ? ones : ~ones;
-                }
-                unsigned int pos = 0;
-                if (act) pos = S.hist[d][wid] + __popc(peers & lt_mask);
-                __syncwarp();
-                if (act && lane == __ffs(peers) - 1) S.hist[d][wid] += __popc(peers);
-                if (act) {
-                    S.key[cur ^ 1][pos] = key;
-                    S.val[cur ^ 1][pos] = S.val[cur][i];
-                }
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-        cur ^= 1;
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        if (tid + j * SORT_THREADS < n) atomicAdd(&S.bin[(d[j] - kmin) >> sh], 1u);
     }
-    // runs of equal compressed key: up to FIX_RUN keys are ordered by
-    // (depth bits, slot) by the thread that finds the run (insertion sort);
-    // a longer run (many equal or nearly equal depths) is recorded and then
-    // sorted by the whole block, so no thread sorts thousands of keys alone
-    // (the histogram is free after the passes and holds the list)
-    unsigned int *nlong = &S.hist[0][0], *lrun = &S.hist[0][1];
-    if (threadIdx.x == 0) *nlong = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += SORT_THREADS) {
-        const unsigned int c = (S.key[cur][i] - kmin) >> shift;
-        if ((i == 0 || ((S.key[cur][i - 1] - kmin) >> shift) != c) && i + 1 < n &&
-            ((S.key[cur][i + 1] - kmin) >> shift) == c) {
-            int e = i + 1;
-            while (e < n && ((S.key[cur][e] - kmin) >> shift) == c) ++e;
-            if (e - i > FIX_RUN) {
-                const unsigned int q = atomicAdd(nlong, 1u);   // at most n / (FIX_RUN + 1) runs
-                lrun[2 * q] = (unsigned int)i;
-                lrun[2 * q + 1] = (unsigned int)(e - i);
-                continue;
-            }
-            for (int a = i + 1; a < e; ++a) {
-                const unsigned int ka = S.key[cur][a], va = S.val[cur][a];
-                int b = a - 1;
-                while (b >= i && (S.key[cur][b] > ka || (S.key[cur][b] == ka && S.val[cur][b] > va))) {
-                    S.key[cur][b + 1] = S.key[cur][b];
-                    S.val[cur][b + 1] = S.val[cur][b];
-                    --b;
-                }
-                S.key[cur][b + 1] = ka;
-                S.val[cur][b + 1] = va;
-            }
+    {
+        // first bucket of each bin, neighbouring bins per thread; the buckets'
+        // counters start at zero
+        unsigned int c[SORT_BIN_PER], sum = 0u;
+#pragma unroll
+        for (int k = 0; k < SORT_BIN_PER; ++k) {
+            c[k] = S.bin[SORT_BIN_PER * tid + k];
+            sum += c[k];
+        }
+        unsigned int first = block_excl_sum(S, sum);
+#pragma unroll
+        for (int k = 0; k < SORT_BIN_PER; ++k) {
+            S.bin[SORT_BIN_PER * tid + k] = first;
+            first += c[k];
+        }
+        if (tid == SORT_THREADS - 1) S.bin[SORT_BINS] = first;
+        for (int i = tid; 4 * i <= n; i += SORT_THREADS) S.bucket4[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    __syncthreads();
+    // bucket and arrival rank of each key (two 16-bit halves of at[]): a bin of
+    // c keys is cut into c equal steps of the bits below the bin's
+#pragma unroll
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        if (tid + j * SORT_THREADS < n) {
+            const unsigned int k = d[j] - kmin, b = k >> sh, f = S.bin[b], c = S.bin[b + 1] - f;
+            const unsigned int q = f + (sh ? __umulhi(k << (32 - sh), c) : 0u);
+            at[j] = q << 16 | atomicAdd(bucket + q, 1u);
         }
     }
     __syncthreads();
-    const unsigned int n_long = *nlong;
+    {
+        // first position of each bucket, neighbouring buckets per thread: as few
+        // groups of four each as the tile needs
+        const int groups = (n / 4 + SORT_THREADS) / SORT_THREADS;   // (buckets 0 .. n)
+        unsigned int sum = 0u;
+        for (int gq = 0; gq < groups; ++gq) {
+            const int i = groups * tid + gq;
+            if (4 * i <= n) {
+                const uint4 c = S.bucket4[i];
+                sum += c.x + c.y + c.z + c.w;
+            }
+        }
+        unsigned int first = block_excl_sum(S, sum);
+        for (int gq = 0; gq < groups; ++gq) {
+            const int i = groups * tid + gq;
+            if (4 * i > n) break;
+            const uint4 c4 = S.bucket4[i];
+            const unsigned int c[4] = {c4.x, c4.y, c4.z, c4.w};
+            unsigned int p[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                p[k] = first;
+                first += c[k];
+                if (c[k] > FIX_RUN) {
+                    const unsigned int q = atomicAdd(&S.nlong, 1u);   // at most n / (FIX_RUN + 1)
+                    S.lrun[2 * q] = p[k];
+                    S.lrun[2 * q + 1] = c[k];
+                }
+            }
+            S.bucket4[i] = make_uint4(p[0], p[1], p[2], p[3]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        if (tid + j * SORT_THREADS < n) {
+            const unsigned int pos = bucket[at[j] >> 16] + (at[j] & 0xffffu);
+            S.key[pos] = d[j];
+            S.val[pos] = v[j];
+        }
+    }
+    __syncthreads();
+    // the place of each key in its bucket: the number of smaller keys there
+#pragma unroll
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        if (tid + j * SORT_THREADS < n) {
+            const unsigned int q = at[j] >> 16, p0 = bucket[q], p1 = bucket[q + 1];
+            at[j] = 0xffffffffu;   // alone in its bucket, or in one sorted below
+            if (p1 - p0 > 1u && p1 - p0 <= (unsigned int)FIX_RUN) {
+                unsigned int less = p0;
+                for (unsigned int i = p0; i < p1; ++i) {
+                    const unsigned int ki = S.key[i];
+                    less += ki < d[j] || (ki == d[j] && S.val[i] < v[j]);
+                }
+                at[j] = less;
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        if (tid + j * SORT_THREADS < n && at[j] != 0xffffffffu) {
+            S.key[at[j]] = d[j];
+            S.val[at[j]] = v[j];
+        }
+    }
+    __syncthreads();
+    // buckets of many keys (many equal or nearly equal depths): by the whole block
+    const unsigned int n_long = S.nlong;
     for (unsigned int q = 0; q < n_long; ++q)
-        block_sort_run(S.key[cur] + lrun[2 * q], S.val[cur] + lrun[2 * q], (int)lrun[2 * q + 1]);
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += SORT_THREADS) {
-        const unsigned int v = S.val[cur][i];
-        keys[st + i] = ((unsigned long long)S.key[cur][i] << 32) | v;
-        if (write_ids) ids[st + i] = v;
+        block_sort_run(S.key + S.lrun[2 * q], S.val + S.lrun[2 * q], (int)S.lrun[2 * q + 1]);
+#pragma unroll
+    for (int j = 0; j < SORT_PER; ++j) {
+        if (j * SORT_THREADS >= n) break;
+        const int i = tid + j * SORT_THREADS;
+        if (i < n) {
+            const unsigned int w = S.val[i];
+            keys[st + i] = ((unsigned long long)S.key[i] << 32) | w;
+            if (write_ids) ids[st + i] = w;
+        }
     }
     __syncthreads();
 }
@@ -549,27 +585,29 @@ __device__ void block_merge(const unsigned long long *a, int na, const unsigned 
     }
 }
 
-// Sort a segment longer than SORT_CAP whose keys are in tmp[st .. st+n):
-// chunks of SORT_CAP sorted on chip into keys, then pairwise merges
-// (ping-pong between keys and tmp over the same index range); the result,
-// with its ids, ends in keys.
-__device__ void sort_segment_merge(SortSmem &S, unsigned long long *keys, unsigned long long *tmp,
-                                   unsigned int *__restrict__ ids, int st, int n) {
-    for (int c = 0; c < n; c += SORT_CAP) radix_sort_tile(S, tmp, keys, ids, st + c, min(SORT_CAP, n - c), false);
-    unsigned long long *src = keys + st, *dst = tmp + st;
+// Sort the segment [st, st + n) of src (keys itself, or tmp) into keys, with its
+// ids. Longer than SORT_CAP (src must be tmp): chunks of SORT_CAP sorted on chip
+// into keys, then pairwise merges (ping-pong between keys and tmp over the same
+// index range), the result ending in keys. Whole block.
+__device__ __forceinline__ void sort_segment(SortSmem &S, const unsigned long long *src, unsigned long long *keys,
+                                             unsigned long long *tmp, unsigned int *__restrict__ ids, int st, int n) {
+    const bool chunks = n > SORT_CAP;
+    for (int c = 0; c < n; c += SORT_CAP) sort_on_chip(S, src, keys, ids, st + c, min(SORT_CAP, n - c), !chunks);
+    if (!chunks) return;
+    unsigned long long *from = keys + st, *to = tmp + st;
     for (int w = SORT_CAP; w < n; w <<= 1) {
         for (int m = 0; m < n; m += 2 * w) {
             const int na = min(w, n - m), nb = max(0, min(w, n - m - w));
-            block_merge(src + m, na, src + m + na, nb, dst + m);
+            block_merge(from + m, na, from + m + na, nb, to + m);
         }
         __syncthreads();
-        unsigned long long *t = src;
-        src = dst;
-        dst = t;
+        unsigned long long *t = from;
+        from = to;
+        to = t;
     }
     for (int i = threadIdx.x; i < n; i += SORT_THREADS) {
-        const unsigned long long k = src[i];
-        if (src != keys + st) keys[st + i] = k;
+        const unsigned long long k = from[i];
+        if (from != keys + st) keys[st + i] = k;
         ids[st + i] = (unsigned int)(k & 0xffffffffu);
     }
     __syncthreads();
@@ -822,53 +860,46 @@ __global__ void __launch_bounds__(SORT_THREADS, 3) k_sort_tiles(const Launch L, 
         __syncthreads();
         const int item = S.item;
         __syncthreads();
+        // the item's segments: a run, a tile, or the runs of bins of a large tile
+        // that was left whole, which fit on chip (but for a single larger bin)
+        const unsigned long long *src = keys_tmp;
+        int st, len, bin0 = 256, base = 0;
         if (item < R) {
-            const int st = runq[2 * item], len = runq[2 * item + 1];
-            if (len == 0) continue;   // a slot of a reservation that did not fit
-            if (len == 1) {
-                if (threadIdx.x == 0) {
-                    const unsigned long long k = keys_tmp[st];
-                    keys[st] = k;
-                    ids[st] = (unsigned int)(k & 0xffffffffu);
-                }
-                continue;
+            st = runq[2 * item];
+            len = runq[2 * item + 1];   // (0: a slot of a reservation that did not fit)
+        } else {
+            if (item - R >= L.n_tiles) break;
+            const int t = order[item - R];
+            const int2 r = ranges[t];
+            st = r.x;
+            len = r.y - r.x;
+            if (len <= SORT_CAP) {
+                src = keys;
+            } else {
+                if (flags[t] < 0) continue;   // split: its runs were items of this queue
+                partition_tile<SORT_THREADS>(keys, keys_tmp, st, len, S.bin, S.moff, S.part, &S.kmin, &S.kmax);
+                base = st;
+                bin0 = 0;
+                len = 0;
             }
-            if (len <= SORT_CAP) radix_sort_tile(S, keys_tmp, keys, ids, st, len, true);
-            else sort_segment_merge(S, keys, keys_tmp, ids, st, len);
-            continue;
         }
-        if (item - R >= L.n_tiles) break;
-        const int t = order[item - R];
-        const int2 r = ranges[t];
-        const int n = r.y - r.x;
-        if (n <= 1) {
-            if (n == 1 && threadIdx.x == 0) ids[r.x] = (unsigned int)(keys[r.x] & 0xffffffffu);
-            continue;
-        }
-        if (n <= SORT_CAP) {
-            radix_sort_tile(S, keys, keys, ids, r.x, n, true);
-            continue;
-        }
-        if (flags[t] < 0) continue;   // split: its runs were items of this queue
-        // a large tile left whole: partition, then sort runs of bins that fit
-        // on chip one after another (a single bin larger than that takes the
-        // chunk-and-merge path). The result is the same (depth, slot) order.
-        partition_tile<SORT_THREADS>(keys, keys_tmp, r.x, n, &S.hist[0][0], S.moff, S.part, &S.kmin, &S.kmax);
-        for (int b0 = 0; b0 < 256;) {
-            const int b1 = run_end(S.moff, b0, SORT_CAP);
-            const int s0 = (int)S.moff[b0], len = (int)(S.moff[b1] - S.moff[b0]);
-            if (len == 1 && threadIdx.x == 0) {
-                const unsigned long long k = keys_tmp[r.x + s0];
-                keys[r.x + s0] = k;
-                ids[r.x + s0] = (unsigned int)(k & 0xffffffffu);
-            } else if (len > 1 && len <= SORT_CAP) {
-                radix_sort_tile(S, keys_tmp, keys, ids, r.x + s0, len, true);
-            } else if (len > SORT_CAP) {
-                sort_segment_merge(S, keys, keys_tmp, ids, r.x + s0, len);
+        for (;;) {
+            if (bin0 < 256) {
+                const int bin1 = run_end(S.moff, bin0, SORT_CAP);
+                st = base + (int)S.moff[bin0];
+                len = (int)(S.moff[bin1] - S.moff[bin0]);
+                bin0 = bin1;
             }
-            __syncthreads();
-            b0 = b1;
+            if (len > 1) {
+                sort_segment(S, src, keys, keys_tmp, ids, st, len);
+            } else if (len == 1 && threadIdx.x == 0) {
+                const unsigned long long k = src[st];
+                keys[st] = k;
+                ids[st] = (unsigned int)(k & 0xffffffffu);
+            }
+            if (bin0 >= 256) break;
         }
+        __syncthreads();   // moff has been read
     }
 }
 
