@@ -5,13 +5,19 @@
 //
 // One kernel does the forward and the backward for a 32x32 output tile and
 // all three channels: it stages x and y with a 10-pixel halo in shared
-// memory, blurs x, y, x^2, y^2, xy (separable: a horizontal then a vertical
-// 11-tap pass) over the tile plus a 5-pixel halo, forms SSIM and the three
+// memory, blurs x, y, x^2 + y^2, xy (separable: a horizontal then a vertical
+// 11-tap pass) over the tile plus a 5-pixel halo (SSIM and its derivatives
+// need the two variances only as their sum), forms SSIM and the three
 // per-pixel derivative fields a = dS/dmu_x, b = dS/dE[x^2], c = dS/dE[xy]
 // there, blurs those over the tile, and writes
 //   dL/dx = (1 - lambda) sign(x - y) / n - lambda / n (G a + 2 x G b + y G c).
 // Every pass keeps a run of outputs per thread in registers so that each
 // staged value is read from shared memory once per run, not once per tap.
+// Bound by instruction issue, with a barrier after each of the five passes: it
+// needs several blocks per SM to cover them, so a, b, c take the staged inputs'
+// place (the centre pixels are read again from the caches) and registers are
+// capped for four blocks. Two 1237x822 images: 138 us (three blocks 142, two
+// 158); 174 us with five blurs, its own room for a, b, c and two blocks per SM.
 #include "gs_common.cuh"
 
 namespace gsk {
@@ -34,17 +40,18 @@ struct SsimLaunch {
 };
 
 struct SsimSmem {
-    float x[SS_IN][SS_IN];
-    float y[SS_IN][SS_IN];
     union {
-        float h1[5][SS_IN][SS_S1];   // horizontal blurs of x, y, x^2, y^2, xy
-        float h2[3][SS_S1][SS_T];    // horizontal blurs of a, b, c
+        float xy[2][SS_IN][SS_IN];    // x, y
+        float abc[3][SS_S1][SS_S1];
+    } in;
+    union {
+        float h1[4][SS_IN][SS_S1];    // horizontal blurs of x, y, x^2 + y^2, xy
+        float h2[3][SS_S1][SS_T];     // horizontal blurs of a, b, c
     } u;
-    float abc[3][SS_S1][SS_S1];
     float red[2][SS_THREADS / 32];
 };
 
-__global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, const float *__restrict__ image,
+__global__ void __launch_bounds__(SS_THREADS, 4) k_l1_dssim(const SsimLaunch L, const float *__restrict__ image,
                                                             const float *__restrict__ target, float *__restrict__ grad,
                                                             float *loss) {
     extern __shared__ __align__(16) unsigned char ss_raw[];
@@ -70,37 +77,36 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
             const int r = i / SS_IN, c = i % SS_IN;
             const int gy = oy - 2 * SS_R + r, gx = ox - 2 * SS_R + c;
             const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
-            sm.x[r][c] = in ? X[(long long)gy * W + gx] : 0.f;
-            sm.y[r][c] = in ? Y[(long long)gy * W + gx] : 0.f;
+            sm.in.xy[0][r][c] = in ? X[(long long)gy * W + gx] : 0.f;
+            sm.in.xy[1][r][c] = in ? Y[(long long)gy * W + gx] : 0.f;
         }
         __syncthreads();
         // horizontal pass: 52 rows x 42 columns, runs of 7 columns per thread
         constexpr int RUN1 = 7;
         for (int i = tid; i < SS_IN * (SS_S1 / RUN1); i += SS_THREADS) {
             const int r = i / (SS_S1 / RUN1), c0 = (i % (SS_S1 / RUN1)) * RUN1;
-            float a[5][RUN1];
+            float a[4][RUN1];
 #pragma unroll
-            for (int q = 0; q < 5; ++q)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
                 for (int j = 0; j < RUN1; ++j) a[q][j] = 0.f;
 #pragma unroll
             for (int k = 0; k < RUN1 + 2 * SS_R; ++k) {
-                const float xv = sm.x[r][c0 + k], yv = sm.y[r][c0 + k];
-                const float xx = xv * xv, yy = yv * yv, xy = xv * yv;
+                const float xv = sm.in.xy[0][r][c0 + k], yv = sm.in.xy[1][r][c0 + k];
+                const float sq = fmaf(xv, xv, yv * yv), xy = xv * yv;
 #pragma unroll
                 for (int j = 0; j < RUN1; ++j) {
                     const int t = k - j;
                     if (t >= 0 && t <= 2 * SS_R) {
                         a[0][j] = fmaf(g[t], xv, a[0][j]);
                         a[1][j] = fmaf(g[t], yv, a[1][j]);
-                        a[2][j] = fmaf(g[t], xx, a[2][j]);
-                        a[3][j] = fmaf(g[t], yy, a[3][j]);
-                        a[4][j] = fmaf(g[t], xy, a[4][j]);
+                        a[2][j] = fmaf(g[t], sq, a[2][j]);
+                        a[3][j] = fmaf(g[t], xy, a[3][j]);
                     }
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 5; ++q)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
                 for (int j = 0; j < RUN1; ++j) sm.u.h1[q][r][c0 + j] = a[q][j];
         }
@@ -108,15 +114,15 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
         // vertical pass over the 42x42 region, runs of 7 rows: SSIM and a, b, c
         for (int i = tid; i < SS_S1 * (SS_S1 / RUN1); i += SS_THREADS) {
             const int c = i % SS_S1, r0 = (i / SS_S1) * RUN1;
-            float a[5][RUN1];
+            float a[4][RUN1];
 #pragma unroll
-            for (int q = 0; q < 5; ++q)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
                 for (int j = 0; j < RUN1; ++j) a[q][j] = 0.f;
 #pragma unroll
             for (int k = 0; k < RUN1 + 2 * SS_R; ++k) {
 #pragma unroll
-                for (int q = 0; q < 5; ++q) {
+                for (int q = 0; q < 4; ++q) {
                     const float hv = sm.u.h1[q][r0 + k][c];
 #pragma unroll
                     for (int j = 0; j < RUN1; ++j) {
@@ -133,9 +139,9 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
                 float da = 0.f, db = 0.f, dc = 0.f;
                 if (gy >= 0 && gy < H && gx >= 0 && gx < W) {
                     const float mx = a[0][j], my = a[1][j];
-                    const float sxx = a[2][j] - mx * mx, syy = a[3][j] - my * my, sxy = a[4][j] - mx * my;
+                    const float m2 = mx * mx + my * my, sxy = a[3][j] - mx * my;
                     const float l1 = 2.f * mx * my + SS_C1, l2 = 2.f * sxy + SS_C2;
-                    const float d1 = mx * mx + my * my + SS_C1, d2 = sxx + syy + SS_C2;
+                    const float d1 = m2 + SS_C1, d2 = (a[2][j] - m2) + SS_C2;
                     const float rd1 = 1.f / d1, rd2 = 1.f / d2, rq = rd1 * rd2;
                     const float S = l1 * l2 * rq;
                     // dS/dmu_x with E[x^2] and E[xy] held fixed, written without
@@ -146,9 +152,9 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
                     dc = 2.f * l1 * rq;
                     if (r >= SS_R && r < SS_R + SS_T && c >= SS_R && c < SS_R + SS_T) acc_s += S;
                 }
-                sm.abc[0][r][c] = da;
-                sm.abc[1][r][c] = db;
-                sm.abc[2][r][c] = dc;
+                sm.in.abc[0][r][c] = da;
+                sm.in.abc[1][r][c] = db;
+                sm.in.abc[2][r][c] = dc;
             }
         }
         __syncthreads();
@@ -165,7 +171,7 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
             for (int k = 0; k < RUN2 + 2 * SS_R; ++k) {
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    const float hv = sm.abc[q][r][c0 + k];
+                    const float hv = sm.in.abc[q][r][c0 + k];
 #pragma unroll
                     for (int j = 0; j < RUN2; ++j) {
                         const int t = k - j;
@@ -204,7 +210,7 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
             for (int j = 0; j < RUN2; ++j) {
                 const int gy = oy + r0 + j;
                 if (gy < H && gx < W) {
-                    const float xv = sm.x[2 * SS_R + r0 + j][2 * SS_R + c], yv = sm.y[2 * SS_R + r0 + j][2 * SS_R + c];
+                    const float xv = X[(long long)gy * W + gx], yv = Y[(long long)gy * W + gx];
                     const float d = xv - yv;
                     acc_l1 += fabsf(d);
                     const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
@@ -234,14 +240,15 @@ __global__ void __launch_bounds__(SS_THREADS, 2) k_l1_dssim(const SsimLaunch L, 
         }
         atomicAdd(&loss[1], l * L.inv_n);
         atomicAdd(&loss[2], s * L.inv_n);
+        // the last block (counted in loss[0], zero before) forms the loss
+        __threadfence();
+        if (atomicAdd(reinterpret_cast<unsigned int *>(loss), 1u) == gridDim.x - 1) {
+            __threadfence();
+            const float l1 = __ldcg(loss + 1), dssim = 1.f - __ldcg(loss + 2);
+            loss[2] = dssim;
+            loss[0] = (1.f - L.lambda) * l1 + L.lambda * dssim;
+        }
     }
-}
-
-// loss = {total, mean L1, 1 - mean SSIM} from the accumulated means
-__global__ void k_l1_dssim_final(float *loss, float lambda) {
-    const float l1 = loss[1], dssim = 1.f - loss[2];
-    loss[2] = dssim;
-    loss[0] = (1.f - lambda) * l1 + lambda * dssim;
 }
 
 int launch_l1_dssim(const int *W, const int *H, int n_views, const float *image, const float *target, float lambda,
@@ -270,14 +277,11 @@ int launch_l1_dssim(const int *W, const int *H, int n_views, const float *image,
     L.lambda = lambda;
     L.inv_n = pix > 0 ? (float)(1.0 / (double)pix) : 0.f;
     if (cudaMemsetAsync(loss, 0, 3 * sizeof(float), st) != cudaSuccess) return GS_ERR_CUDA;
-    if (tiles > 0) {
-        const size_t smem = sizeof(SsimSmem);
-        if (cudaFuncSetAttribute(k_l1_dssim, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return GS_ERR_CUDA;
-        k_l1_dssim<<<(unsigned)tiles, SS_THREADS, smem, st>>>(L, image, target, grad, loss);
-        if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-    }
-    k_l1_dssim_final<<<1, 1, 0, st>>>(loss, lambda);
+    const size_t smem = sizeof(SsimSmem);
+    if (cudaFuncSetAttribute(k_l1_dssim, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return GS_ERR_CUDA;
+    // (views are at least 1x1: there is a tile)
+    k_l1_dssim<<<(unsigned)tiles, SS_THREADS, smem, st>>>(L, image, target, grad, loss);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 

@@ -43,7 +43,7 @@ class GraphStep:
     # project 1, bin/sort 5 (count, scan, scatter, split, sort), render 1, the
     # zeroing of the backward's accumulators 1 (a kernel with overlap_prev),
     # raster bwd 1, projection bwd 1, pose 1; the L1 loss is part of the raster
-    # backward, the L1 + D-SSIM loss adds 2 kernels
+    # backward, the L1 + D-SSIM loss adds 1 kernel
     KERNELS_FIXED = 11
     # the calls of a step, in order (the stages of run()'s events)
     STAGES = {"l1": ("gs_project", "gs_bin_sort", "gs_render_fwd", "gs_rasterize_bwd_l1", "gs_project_bwd",
@@ -57,10 +57,10 @@ class GraphStep:
 
     def kernels_per_step(self) -> int:
         """Kernels of this library that one step launches: the fixed eleven, the
-        D-SSIM loss kernels, and, when the image has fewer than 16 tiles per
+        D-SSIM loss kernel, and, when the image has fewer than 16 tiles per
         SM, the tile orderings by replay length that the raster forward (from
         the previous forward's record) and the raster backward run first."""
-        loss = 0 if self.loss_kind == "l1" else 2
+        loss = 0 if self.loss_kind == "l1" else 1
         sms = torch.cuda.get_device_properties(self.g.means.device).multi_processor_count
         order = 2 if 0 < self.bins.n_tiles < 16 * sms else 0
         return self.KERNELS_FIXED + loss + order
