@@ -623,12 +623,16 @@ int launch_zero_accumulators(float *grad2d, long long n_floats, float *loss, cud
 
 // Resident blocks per SM of a raster kernel at the launch's block and
 // dynamic shared-memory size (cached per batch size; the attribute that
-// allows more than 48 KB of dynamic shared memory is set on first use).
+// allows more dynamic shared memory than so far is set on first use).
 template <typename K>
 static int raster_blocks_per_sm(K kernel, int threads, size_t smem, int batch, int *cache) {
     if (!cache[batch]) {
         int n = 0;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        // the limit is only ever raised: a smaller batch used later must not take
+        // it from a larger one used before
+        cudaFuncAttributes fa;
+        const bool below = cudaFuncGetAttributes(&fa, kernel) == cudaSuccess && fa.maxDynamicSharedSizeBytes < (int)smem;
+        if ((below && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess || n < 1) {
             cudaGetLastError();   // the launch itself reports a size that cannot run
             n = 1;
