@@ -87,7 +87,8 @@ typedef struct gs_config {
                              tensor copies where the layout allows; 0: per-thread loads and stores. The
                              results are the same bit for bit. */
     int fwd_batch;        /* [2] Gaussians each thread stages per shared-memory batch in gs_render_fwd:
-                             1, 2 or 4 (a batch is fwd_batch x tile_w x tile_h / 2 Gaussians) */
+                             1, 2 or 4 (a batch is fwd_batch x threads Gaussians; a block has a thread
+                             per two pixels of its tile, or of a 16x16 part of a tile above 256) */
     int bwd_batch;        /* [1] the same for gs_rasterize_bwd: 1 or 2. Neither changes the image; the
                              2D gradients change only in the order of their float additions. */
     int overlap_prev;     /* [0] nonzero: gs_rasterize_bwd(_l1) and the one-view gs_project_bwd with
@@ -135,7 +136,7 @@ typedef struct gs_bins {
     uint64_t *keys_tmp;   /* [capacity] scratch for tiles too large for on-chip sorting */
     int32_t *tile_order;  /* [T] work order: tiles by decreasing instance count */
     int32_t *tile_scratch;/* [5T] scratch (per-tile counters, then the runs of large tiles that
-                             are sorted in pieces) */
+                             are sorted in pieces, and the blocks' parts of the folded L1 loss) */
     int32_t *counters;    /* [GS_NUM_COUNTERS] scratch; counters[0] = instances after the call;
                              int64 at counters+8: pixel-Gaussian pairs evaluated by gs_render_fwd,
                              +10: composited by it, +12/+14: the same for gs_rasterize_bwd */

@@ -63,6 +63,7 @@ enum {
     CNT_Q_FWD = 2,       // work queue heads
     CNT_Q_BWD = 3,
     CNT_Q_SORT = 4,
+    CNT_L1_DONE = 4,     // (after the sort) blocks of the raster backward whose part of the loss is written
     CNT_RUN_RES = 5,     // runs of split large tiles listed for the sort
     CNT_MAX_TILE = 6,    // largest per-tile count
     CNT_Q_SPLIT = 7      // queue head of the large-tile split

@@ -8,12 +8,13 @@
 //   the Gaussian that would bring T (1 - alpha) below t_min is not composited
 //   and the pixel stops.
 //
-// Both kernels are persistent: blocks pull tiles from an atomic queue over
-// tile_order (largest tiles first). Each thread owns two pixels and each warp
-// an 8x8-pixel patch of the tile; a tile's instances are staged through
-// shared memory in batches (the number per thread chosen at launch: by
-// default two in the forward, one in the backward), and a warp skips every
-// staged Gaussian that cannot reach its patch.
+// Both kernels are persistent: blocks pull regions of tiles from an atomic
+// queue over tile_order (largest tiles first). A region is the tile, or for
+// 32x32 and 32x16 tiles one of its 16x16 quarters or halves (see Region).
+// Each thread owns two pixels and each warp an 8x8-pixel patch of the region; a
+// tile's instances are staged through shared memory in batches (the number per
+// thread chosen at launch: by default two in the forward, one in the backward),
+// and a warp skips every staged Gaussian that cannot reach its patch.
 //
 // The backward does not store or replay transmittance: it walks the same list
 // front to back with bit-identical arithmetic (explicit-rounding intrinsics,
@@ -21,12 +22,14 @@
 // everything behind Gaussian i from the forward image,
 //   S_i = sum_{j>i} c_j alpha_j T_j + T_final bg = image - sum_{j<=i} c_j alpha_j T_j,
 // so that dL/dalpha_i = T_i (c_i . g) - (S_i . g) / (1 - alpha_i).
-// Per-Gaussian gradients (mean2D, 2D covariance, opacity, colour) are summed over a
-// warp through a shared-memory transpose: a warp writes the 9 values of up to
-// three consecutive visits as rows of a per-warp buffer (one column per lane),
-// then 27 lanes each add one row with 16-byte loads; then over the block in
-// shared memory, and into the per-slot grad2d record with one vector atomic
-// per float4.
+// Per-Gaussian gradients (mean2D, 2D covariance, opacity, colour) are linear in
+// two numbers per pixel, the weight w = alpha T and dp = dL/dalpha o G: a visit
+// only stores these two for its pixels in a per-warp buffer; when eight visits
+// are pending, four lanes per visit add up the moments of dp over the patch and
+// the sums of w times the upstream gradient. The moments are summed over the
+// block in shared memory and turned into the nine gradients once per (region,
+// Gaussian), which go to the per-slot grad2d record with one vector atomic per
+// float4.
 // Both kernels run a thread's two pixels through packed float2 arithmetic
 // (f32x2 fma/mul/add, one instruction for both), branch-free: a pixel that
 // does not composite a Gaussian contributes zeros.
@@ -39,7 +42,7 @@ namespace gsk {
 // half-extents (ext_x, ext_y <= radius, so the test |dx| <= ext_x, |dy| <=
 // ext_y implies the radius gate and rejects only pixels whose alpha is below
 // alpha_min anyway); con = quadratic-form coefficients and opacity; rgb =
-// colour and the slot.
+// colour and the instance's index in the tile lists.
 //
 // The exponent -1/2 d^T conic d is evaluated as the sum of two non-negative
 // terms, -1/2 [A u^2 + dy^2 / c] with u = dx - (b/c) dy and A = c / det (the
@@ -47,15 +50,15 @@ namespace gsk {
 // (a, b, c)). The expanded form A dx^2 + 2B dx dy + C dy^2 cancels badly for
 // elongated Gaussians far along their long axis (a factor ~100 in float32);
 // this one does not, at the same five operations per pixel.
-__device__ __forceinline__ void stage(const float4 *__restrict__ proj, unsigned int slot, float ox, float oy,
-                                      float4 &xy, float4 &con, float4 &rgb) {
+__device__ __forceinline__ void stage(const float4 *__restrict__ proj, unsigned int slot, int index, float ox,
+                                      float oy, float4 &xy, float4 &con, float4 &rgb) {
     const float4 r0 = proj[4ull * slot];
     const float4 r1 = proj[4ull * slot + 1];
     const float4 r2 = proj[4ull * slot + 2];
     const float4 r3 = proj[4ull * slot + 3];
     xy = make_float4(__fadd_rn(__fsub_rn(r0.x, ox), r3.x), __fadd_rn(__fsub_rn(r0.y, oy), r3.y), r0.z, r0.w);
     con = r1;   // the conic in the staged form, written by the projection
-    rgb = make_float4(r2.x, r2.y, r2.z, __uint_as_float(slot));
+    rgb = make_float4(r2.x, r2.y, r2.z, __int_as_float(index));
 }
 
 // alpha of a staged Gaussian at a pixel (the forward and the backward share
@@ -80,37 +83,59 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+// The raster kernels' unit of work: RW x RH pixels of a TW x TH tile, BS =
+// RW RH / 2 threads. Tiles of more than 256 pixels are walked in 16x16 parts by
+// 128-thread blocks that each go through the tile's list and stage only what
+// reaches their part. The barriers around a batch make a block's warps wait
+// for the one with the most visits: with a 512-thread block on a 32x32 tile of
+// the 1M-Gaussian view the slowest warp had 1.51 times the mean warp's visits
+// per batch (1.34 per tile), with 16x16 parts 1.24 (1.15). Testing a Gaussian
+// once per part costs a few instructions against the ~100 of a visit, and the
+// coarser tiles keep binning and the sort cheap. Smaller parts would balance
+// better still, but each adds its own sum to a Gaussian's gradient, in float32.
+// With the sums over pending visits below: backward 309 -> 267 us on the 1M
+// view; steps 687 -> 668 us (1M view), 4169 -> 4062 (16-view orbit), 6329 -> 6070
+// (16 uneven views).
+template <int TW, int TH>
+struct Region {
+    static constexpr bool SPLIT = TW * TH > 256;
+    static constexpr int RW = SPLIT ? 16 : TW, RH = SPLIT ? 16 : TH;
+    static constexpr int SX = TW / RW, PARTS = SX * (TH / RH);
+    static constexpr int BS = RW * RH / 2, WARPS = BS / 32;
+};
+
 struct TileInfo {
     int view;
     int px, py0;      // this thread's pixels: (px, py0) and (px, py0 + 4)
     float ox, oy;     // origin of the enclosing 32x32-pixel block
     float pcx, pcy0;  // pixel centres relative to the block origin (second pixel: pcy0 + 4)
-    float tbx, tby;   // tile origin relative to the block origin
+    float tbx, tby;   // region origin relative to the block origin
     bool in0, in1;    // pixels inside the image
 };
 
-// Pixels: warp w covers the 8x8 patch (w % (TW/8), w / (TW/8)) of the tile;
+// Pixels: warp w covers the 8x8 patch (w % (RW/8), w / (RW/8)) of the region;
 // lane l owns column l & 7 and rows (l >> 3) and (l >> 3) + 4 of the patch.
 // Positions are relative to the enclosing 32x32-pixel block (every supported
 // tile nests in one), so a pixel's arithmetic is the same for every tile
 // shape and the image is bit-identical across shapes.
 template <int TW, int TH>
-__device__ __forceinline__ TileInfo tile_info(const Launch &L, int tile) {
+__device__ __forceinline__ TileInfo tile_info(const Launch &L, int tile, int part) {
+    using R = Region<TW, TH>;
     TileInfo ti;
     ti.view = view_of_tile(L, tile);
     const ViewDesc &vd = L.v[ti.view];
     const int lt = tile - vd.tile_base;
-    const int tx = lt % vd.Gx, ty = lt / vd.Gx;
+    const int rx = (lt % vd.Gx) * TW + (part % R::SX) * R::RW, ry = (lt / vd.Gx) * TH + (part / R::SX) * R::RH;
     const int w = (int)threadIdx.x >> 5, l = (int)threadIdx.x & 31;
-    ti.px = tx * TW + (w % (TW / 8)) * 8 + (l & 7);
-    ti.py0 = ty * TH + (w / (TW / 8)) * 8 + (l >> 3);
-    const int bx = (tx * TW) & ~31, by = (ty * TH) & ~31;
+    ti.px = rx + (w % (R::RW / 8)) * 8 + (l & 7);
+    ti.py0 = ry + (w / (R::RW / 8)) * 8 + (l >> 3);
+    const int bx = rx & ~31, by = ry & ~31;
     ti.ox = (float)bx;
     ti.oy = (float)by;
     ti.pcx = (float)(ti.px - bx) + 0.5f;
     ti.pcy0 = (float)(ti.py0 - by) + 0.5f;
-    ti.tbx = (float)(tx * TW - bx);
-    ti.tby = (float)(ty * TH - by);
+    ti.tbx = (float)(rx - bx);
+    ti.tby = (float)(ry - by);
     ti.in0 = ti.px < vd.W && ti.py0 < vd.H;
     ti.in1 = ti.px < vd.W && ti.py0 + 4 < vd.H;
     return ti;
@@ -125,10 +150,10 @@ __device__ __forceinline__ TileInfo tile_info(const Launch &L, int tile) {
 //    most Ah umin^2 + Dh dymin^2, where umin and dymin are the smallest |u|
 //    and |dy| over the patch (u ranges over the patch's dx interval shifted
 //    by beta times its dy interval). A 1e-3 margin keeps the test safe.
-template <int TW, int TH>
+template <int RW, int RH>
 __device__ __forceinline__ unsigned int warp_mask(const float4 &xy, const float4 &con, float alpha_min, float tbx,
                                                   float tby) {
-    constexpr int WX = TW / 8, WY = TH / 8;
+    constexpr int WX = RW / 8, WY = RH / 8;
     const float ex = xy.z + 1e-3f, ey = xy.w + 1e-3f;
     const float lim = __log2f(alpha_min / con.w) - 1e-3f;
     float dxlo[WX], dylo[WY], bmin[WY], bmax[WY], dy2[WY];
@@ -170,71 +195,203 @@ __device__ __forceinline__ void count_pairs(int *counters, int at, unsigned int 
     }
 }
 
-// Stage instances [b0, min(b0 + per BS, end)) of a tile: per (1, 2 or 4)
-// per thread, the batch size chosen at launch.
+// One staged Gaussian: its three float4 lie together (48 bytes apart, an odd
+// number of 16-byte bank groups: no conflicts on the stores), so that a visit
+// reads them at one address.
 template <int TW, int TH>
-__device__ __forceinline__ void stage_batch(const Launch &L, const float4 *__restrict__ proj,
-                                            const unsigned int *__restrict__ ids, int b0, int end, int per,
-                                            const TileInfo &ti, float4 *s_xy, float4 *s_con, float4 *s_rgb,
-                                            unsigned int *s_mask) {
-    constexpr int BS = TW * TH / 2;
-    for (int h = 0; h < per; ++h) {
-        const int k = threadIdx.x + h * BS;
-        if (b0 + k < end) {
-            stage(proj, ids[b0 + k], ti.ox, ti.oy, s_xy[k], s_con[k], s_rgb[k]);
-            s_mask[k] = warp_mask<TW, TH>(s_xy[k], s_con[k], L.alpha_min, ti.tbx, ti.tby);
+__device__ __forceinline__ void stage_one(const Launch &L, const float4 *__restrict__ proj,
+                                          const unsigned int *__restrict__ ids, int index, int k, const TileInfo &ti,
+                                          float4 *s_st, unsigned char *s_mask) {
+    float4 xy, con, rgb;
+    stage(proj, ids[index], index, ti.ox, ti.oy, xy, con, rgb);
+    s_st[3 * k] = xy;
+    s_st[3 * k + 1] = con;
+    s_st[3 * k + 2] = rgb;
+    s_mask[k] = (unsigned char)warp_mask<Region<TW, TH>::RW, Region<TW, TH>::RH>(xy, con, L.alpha_min, ti.tbx, ti.tby);
+}
+
+// Stage the next batch of a tile's instances [pos, end) that reach the block's
+// region: at most per BS of them (per: 1, 2 or 4 per thread, the batch size
+// chosen at launch), in list order; pos moves past the last one looked at.
+// Returns their number. With one part per tile every instance is taken (the
+// binning's rectangles already reach the region). With several, each thread
+// first tests the reach boxes of up to PARTS per instances (at most 8), and
+// the ones that overlap the region are packed: (test j, warp) ballots in shared
+// memory, their prefix sums by every warp for itself. Whole block; the staged
+// batch is visible to it when this returns.
+struct Pack {
+    unsigned int ballot[32];   // [test j][warp]
+    int next;
+};
+template <int TW, int TH>
+__device__ __forceinline__ int stage_batch(const Launch &L, const float4 *__restrict__ proj,
+                                           const unsigned int *__restrict__ ids, int &pos, int end, int per,
+                                           const TileInfo &ti, float4 *s_st, unsigned char *s_mask, Pack *pk) {
+    using R = Region<TW, TH>;
+    constexpr int BS = R::BS;
+    if constexpr (R::PARTS == 1) {
+        for (int h = 0; h < per; ++h) {
+            const int k = threadIdx.x + h * BS;
+            if (k < end - pos) stage_one<TW, TH>(L, proj, ids, pos + k, k, ti, s_st, s_mask);
         }
+        const int nb = min(per * BS, end - pos);
+        pos += nb;
+        __syncthreads();
+        return nb;
+    } else {
+        static_assert(8 * R::WARPS <= 32, "one ballot per lane of the prefix sum");
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        const int tests = min(8, R::PARTS * per), cap = per * BS;
+        // the region's box, grown by the part of the mean that the first float4
+        // leaves out and by float rounding
+        const float lx = ti.ox + ti.tbx + 0.5f - 2e-3f, hx = lx + (float)(R::RW - 1) + 4e-3f;
+        const float ly = ti.oy + ti.tby + 0.5f - 2e-3f, hy = ly + (float)(R::RH - 1) + 4e-3f;
+#pragma unroll 4
+        for (int j = 0; j < tests; ++j) {
+            const int at = j * BS + threadIdx.x;
+            bool hit = false;
+            if (at < end - pos) {
+                const float4 r0 = proj[4ull * ids[pos + at]];
+                hit = r0.x + r0.z >= lx && r0.x - r0.z <= hx && r0.y + r0.w >= ly && r0.y - r0.w <= hy;
+            }
+            const unsigned int bal = __ballot_sync(0xffffffffu, hit);
+            if (lane == 0) pk->ballot[j * R::WARPS + wid] = bal;
+        }
+        if (threadIdx.x == 0) pk->next = pos + min(tests * BS, end - pos);
+        __syncthreads();
+        const int n = lane < tests * R::WARPS ? __popc(pk->ballot[lane]) : 0;
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        const int excl = incl - n;
+        for (int j = 0; j < tests; ++j) {
+            const int base = __shfl_sync(0xffffffffu, excl, j * R::WARPS + wid);
+            const unsigned int bal = pk->ballot[j * R::WARPS + wid];
+            const int k = base + __popc(bal & ((1u << lane) - 1u));
+            const int i = pos + j * BS + threadIdx.x;
+            if (bal >> lane & 1u) {
+                if (k < cap) stage_one<TW, TH>(L, proj, ids, i, k, ti, s_st, s_mask);
+                else if (k == cap) pk->next = i;   // the first that did not fit starts the next batch
+            }
+        }
+        __syncthreads();
+        pos = pk->next;
+        return min(total, cap);
     }
 }
 
 // Shared-memory bytes of one staged Gaussian: position, conic and colour
-// (3 x 16 B) and the warp mask; the backward adds the conic's natural-log
-// terms (8 B) and the per-Gaussian gradient sums (9 floats).
-constexpr int FWD_STAGE_BYTES = 52;
-constexpr int BWD_STAGE_BYTES = 96;
-// The backward's per-warp reduction buffer: RED_SLOTS visits x 9 values as
-// rows of 32 lane columns, row pitch RED_PITCH floats (16-byte aligned rows;
-// the 4-float pad puts the 8 lanes of a quarter-warp reading 16 bytes of 8
-// different rows on 8 disjoint groups of 4 banks).
-constexpr int RED_SLOTS = 3;
-constexpr int RED_PITCH = 36;
-constexpr int RED_WARP_FLOATS = RED_SLOTS * 9 * RED_PITCH;
+// (3 x 16 B) and the warp mask (a byte: at most four warps); the backward adds
+// its nine sums.
+constexpr int FWD_STAGE_BYTES = 49;
+constexpr int BWD_STAGE_BYTES = 85;
+// The backward's per-warp buffer: RED_VISITS pending visits of 32 lanes, a
+// float4 (w, dp of the lane's two pixels) each, and the lanes' upstream
+// gradients (a float4 and a float2 each).
+constexpr int RED_VISITS = 8;
+constexpr int RED_WARP_BYTES = RED_VISITS * 32 * 16 + 32 * 24;
+// Threads per SM the backward's registers are capped for: 896 (72 registers, 30 KB
+// of shared memory per 128 threads): 1M view 670 us a step, against 683 with 1,024
+// (64 registers, and six pending visits to fit) and 671 with 768. The one-warp
+// blocks of 8x8 tiles keep more addresses in registers: 640 (96 registers), 24
+// views of three scenes 6.65 ms against 6.97 with 768 and 7.05 with 896.
+constexpr int bwd_blocks(int threads) { return (threads == 32 ? 640 : 896) / threads; }
+
+// Lane l = 8 q + i owns column i and rows q, q + 4 of its patch. Its entry in a
+// row of 32 is at red_at(l), + 4 exchanged in odd visits: the lanes of a
+// quarter-warp that read column i of two visits and four q's then hit the
+// eight 16-byte bank groups once each.
+__device__ __forceinline__ int red_at(int l) { return (l & 24) | ((l & 7) ^ (l >> 3)); }
+
+// Sums over the pending visits' patches, by four lanes per visit: lane 4 s + q
+// of the warp adds up rows q and q + 4 of visit s (lane .x = row q, .y = row
+// q + 4) from its buffer row. u is formed per pixel as in the walk (moments
+// about a fixed point would cancel: u is small on a thin Gaussian's ridge where
+// dx and beta dy are not); dy is constant over a row. The nine sums
+//   sum dp (1, u, dy, u^2, u dy, dy^2), sum w (g_r, g_g, g_b)
+// are folded over the four lanes, each keeping two (lane 0 three), and added to
+// the Gaussian's sums over the block in s_g. k: the staged index of visit s.
+__device__ __forceinline__ void reduce_visits(const float4 *__restrict__ buf, const float4 *__restrict__ g4,
+                                              const float2 *__restrict__ g2, int npend, int k, float px0, float py0,
+                                              const float4 *s_st, float *s_g) {
+    const int lane = threadIdx.x & 31, s = lane >> 2, q = lane & 3;
+    const float4 *row = buf + s * 32 + 8 * q;
+    const int odd = (s & 1) << 2;
+    const float4 xy = s_st[3 * k];
+    const float beta = s_st[3 * k + 1].y;
+    const float y0 = py0 + (float)q;
+    const float2 dy = make_float2(y0 - xy.y, (y0 + 4.f) - xy.y);
+    float2 S0 = make_float2(0.f, 0.f), su = S0, suu = S0, CR = S0, CG = S0, CB = S0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float4 v = row[i ^ (q | odd)];
+        const float4 gv = g4[8 * q + (i ^ q)];
+        const float2 gb = g2[8 * q + (i ^ q)];
+        const float2 w = make_float2(v.x, v.y), dp = make_float2(v.z, v.w);
+        const float dx = (px0 + (float)i) - xy.x;
+        const float2 u = __ffma2_rn(f2(beta), dy, f2(dx));
+        const float2 t = __fmul2_rn(dp, u);
+        S0 = __fadd2_rn(S0, dp);
+        su = __fadd2_rn(su, t);
+        suu = __ffma2_rn(t, u, suu);
+        CR = __ffma2_rn(w, make_float2(gv.x, gv.y), CR);
+        CG = __ffma2_rn(w, make_float2(gv.z, gv.w), CG);
+        CB = __ffma2_rn(w, gb, CB);
+    }
+    const float2 sy = __fmul2_rn(dy, S0), suy = __fmul2_rn(dy, su), syy = __fmul2_rn(dy, sy);
+    const float t[9] = {S0.x + S0.y, su.x + su.y, sy.x + sy.y, suu.x + suu.y, suy.x + suy.y, syy.x + syy.y,
+                        CR.x + CR.y, CG.x + CG.y, CB.x + CB.y};
+    // sums j and j + 4 change hands between the lanes of a pair, then j and
+    // j + 2: lane q ends with sums 4 (q & 1) + (q & 2) + {0, 1}
+    const bool b0 = q & 1, b1 = q & 2;
+    float r[4], z[2], t8 = t[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r[j] = (b0 ? t[j + 4] : t[j]) + __shfl_xor_sync(0xffffffffu, b0 ? t[j] : t[j + 4], 1);
+    t8 += __shfl_xor_sync(0xffffffffu, t8, 1);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) z[j] = (b1 ? r[j + 2] : r[j]) + __shfl_xor_sync(0xffffffffu, b1 ? r[j] : r[j + 2], 2);
+    t8 += __shfl_xor_sync(0xffffffffu, t8, 2);
+    if (s < npend) {
+        float *dst = s_g + 9 * k;
+        float *two = dst + 4 * (q & 1) + (q & 2);
+        atomicAdd(two, z[0]);
+        atomicAdd(two + 1, z[1]);
+        if (q == 0) atomicAdd(dst + 8, t8);
+    }
+}
 
 template <int TW, int TH>
-__global__ void __launch_bounds__(TW * TH / 2) k_render_fwd(const Launch L, const float4 *__restrict__ proj,
-                                                            const int2 *__restrict__ ranges,
-                                                            const unsigned int *__restrict__ ids,
-                                                            const int *__restrict__ order, int *__restrict__ counters,
-                                                            float *__restrict__ image, int *__restrict__ last_contrib,
-                                                            int *__restrict__ tile_work) {
+__global__ void __launch_bounds__(Region<TW, TH>::BS, 1024 / Region<TW, TH>::BS)
+    k_render_fwd(const Launch L, const float4 *__restrict__ proj, const int2 *__restrict__ ranges,
+                 const unsigned int *__restrict__ ids, const int *__restrict__ order, int *__restrict__ counters,
+                 float *__restrict__ image, int *__restrict__ last_contrib, int *__restrict__ tile_work) {
     // the staged batch (L.fwd_batch Gaussians per thread) in dynamic shared memory
-    constexpr int BS = TW * TH / 2;
+    using R = Region<TW, TH>;
+    constexpr int BS = R::BS;
     const int NB = L.fwd_batch * BS;
     extern __shared__ float4 s_dyn[];
-    float4 *s_xy = s_dyn, *s_con = s_xy + NB, *s_rgb = s_con + NB;
-    unsigned int *s_mask = reinterpret_cast<unsigned int *>(s_rgb + NB);
-    __shared__ int s_item, s_end;
+    float4 *s_st = s_dyn;
+    unsigned char *s_mask = reinterpret_cast<unsigned char *>(s_st + 3 * NB);
+    __shared__ int s_item;
+    __shared__ Pack s_pack;
     // the backward's accumulators that follow (zeroed by a programmatic
     // dependent) may be cleared on SMs this kernel leaves in its tail
     launch_dependents();
     const bool abort = counters[CNT_ABORT] != 0;
     const unsigned int wbit = 1u << (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    int prev_tile = -1;   // (thread 0) the tile whose replay length s_end holds
-    if (threadIdx.x == 0) s_end = 0;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(counters + CNT_Q_FWD, 1);
         __syncthreads();
         const int item = s_item;
-        if (tile_work && threadIdx.x == 0) {
-            // every warp has added the previous tile's length before the barrier
-            if (prev_tile >= 0) tile_work[prev_tile] = s_end;
-            s_end = 0;
-        }
         __syncthreads();
-        if (item >= L.n_tiles) break;
-        const int tile = order[item];
-        const TileInfo ti = tile_info<TW, TH>(L, tile);
+        if (item >= L.n_tiles * R::PARTS) break;
+        const int tile = order[item / R::PARTS];
+        const TileInfo ti = tile_info<TW, TH>(L, tile, item % R::PARTS);
         const int2 r = abort ? make_int2(0, 0) : ranges[tile];
         // lane .x = pixel (px, py0), lane .y = pixel (px, py0 + 4)
         float2 T = f2(1.f), CR = f2(0.f), CG = f2(0.f), CB = f2(0.f);
@@ -245,11 +402,9 @@ __global__ void __launch_bounds__(TW * TH / 2) k_render_fwd(const Launch L, cons
         float am0 = ti.in0 ? amin : INF, am1 = ti.in1 ? amin : INF;
         int end0 = r.x, end1 = r.x;   // one past the last composited instance
         const float2 PCY = make_float2(ti.pcy0, ti.pcy0 + 4.f);
-        for (int b0 = r.x; b0 < r.y; b0 += NB) {
+        for (int pos = r.x; pos < r.y;) {
             if (__syncthreads_count(am0 == INF && am1 == INF) == BS) break;
-            stage_batch<TW, TH>(L, proj, ids, b0, r.y, L.fwd_batch, ti, s_xy, s_con, s_rgb, s_mask);
-            __syncthreads();
-            const int nb = min(NB, r.y - b0);
+            const int nb = stage_batch<TW, TH>(L, proj, ids, pos, r.y, L.fwd_batch, ti, s_st, s_mask, &s_pack);
             // the warp walks only the staged Gaussians that may reach its patch:
             // 32 masks per ballot, then the set bits in order
             for (int k0 = 0; k0 < nb; k0 += 32) {
@@ -258,7 +413,7 @@ __global__ void __launch_bounds__(TW * TH / 2) k_render_fwd(const Launch L, cons
                 while (hits) {
                     const int k = k0 + __ffs(hits) - 1;
                     hits &= hits - 1;
-                    const float4 xy = s_xy[k], con = s_con[k];
+                    const float4 xy = s_st[3 * k], con = s_st[3 * k + 1];
                     const float dx = __fsub_rn(ti.pcx, xy.x);
                     const bool col = fabsf(dx) <= xy.z;   // the column gate, shared by both pixels
                     const float2 dy = __fadd2_rn(PCY, f2(-xy.y));
@@ -276,14 +431,15 @@ __global__ void __launch_bounds__(TW * TH / 2) k_render_fwd(const Launch L, cons
                     const bool cp0 = ok0 && !st0, cp1 = ok1 && !st1;
                     am0 = st0 ? INF : am0;
                     am1 = st1 ? INF : am1;
-                    end0 = cp0 ? b0 + k + 1 : end0;
-                    end1 = cp1 ? b0 + k + 1 : end1;
+                    const float4 c = s_st[3 * k + 2];
+                    const int after = __float_as_int(c.w) + 1;
+                    end0 = cp0 ? after : end0;
+                    end1 = cp1 ? after : end1;
                     // weight and transmittance through the composited alpha (alpha, or 0
                     // for a pixel that does not composite: T (1 - 0) is T bit for bit)
                     const float2 ac = make_float2(cp0 ? a0 : 0.f, cp1 ? a1 : 0.f);
                     const float2 w = __fmul2_rn(ac, T);
                     T = __fmul2_rn(T, __fadd2_rn(f2(1.f), make_float2(-ac.x, -ac.y)));
-                    const float4 c = s_rgb[k];
                     CR = __ffma2_rn(f2(c.x), w, CR);
                     CG = __ffma2_rn(f2(c.y), w, CG);
                     CB = __ffma2_rn(f2(c.z), w, CB);
@@ -308,11 +464,9 @@ __global__ void __launch_bounds__(TW * TH / 2) k_render_fwd(const Launch L, cons
             if (last_contrib) last_contrib[vd.pix_base / 3 + (long long)(ti.py0 + 4) * vd.W + ti.px] = end1;
         }
         if (tile_work) {
-            // the backward's replay length of this tile: its pixels' largest
-            // end (written by thread 0 after the next item's barrier)
+            // the tile's replay length: its pixels' largest end
             const int e = __reduce_max_sync(0xffffffffu, max(end0, end1) - r.x);
-            if (lane == 0) atomicMax(&s_end, e);
-            prev_tile = tile;
+            if (lane == 0) atomicMax(tile_work + tile, e);
         }
     }
 }
@@ -324,55 +478,50 @@ __global__ void __launch_bounds__(TW * TH / 2) k_render_fwd(const Launch L, cons
 // is composited, and the warp and the block stop at their pixels' largest
 // end instead of walking on to saturation or the end of the list.
 template <int TW, int TH, bool COUNT, bool LAST>
-__global__ void __launch_bounds__(TW * TH / 2, 1024 / (TW * TH / 2)) k_render_bwd(const Launch L, const float4 *__restrict__ proj,
-                                                            const int2 *__restrict__ ranges,
-                                                            const unsigned int *__restrict__ ids,
-                                                            const int *__restrict__ order, int *__restrict__ counters,
-                                                            const float *__restrict__ image,
-                                                            const float *__restrict__ dL_dimage,
-                                                            const int *__restrict__ last_contrib,
-                                                            float4 *__restrict__ grad2d,
-                                                            const float *__restrict__ l1_target,
-                                                            float *__restrict__ l1_loss, float l1_inv_n) {
-    // dynamic shared memory: the per-warp reduction buffers, then the staged
-    // batch (L.bwd_batch Gaussians per thread): positions, conics, colours,
-    // the conic's A and D (natural-log units), the per-Gaussian gradient sums
-    // (pitch 9, odd: no bank conflicts) and warp masks
-    constexpr int BS = TW * TH / 2;
+__global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>::BS))
+    k_render_bwd(const Launch L, const float4 *__restrict__ proj, const int2 *__restrict__ ranges,
+                 const unsigned int *__restrict__ ids, const int *__restrict__ order, int *__restrict__ counters,
+                 const float *__restrict__ image, const float *__restrict__ dL_dimage,
+                 const int *__restrict__ last_contrib, float4 *__restrict__ grad2d,
+                 const float *__restrict__ l1_target, float *__restrict__ l1_loss, float l1_inv_n,
+                 float *__restrict__ l1_part) {
+    // dynamic shared memory: the per-warp buffers of pending visits and the
+    // lanes' upstream gradients, then the staged batch (L.bwd_batch Gaussians
+    // per thread): positions, conics and colours, the sums over the block
+    // (pitch 9, odd: no bank conflicts) and the warp masks
+    using R = Region<TW, TH>;
+    constexpr int BS = R::BS;
     const int NB = L.bwd_batch * BS;
     extern __shared__ float4 s_dyn[];
-    float *s_red = reinterpret_cast<float *>(s_dyn);
-    float4 *s_xy = s_dyn + (BS / 32) * RED_WARP_FLOATS / 4, *s_con = s_xy + NB, *s_rgb = s_con + NB;
-    float2 *s_ad = reinterpret_cast<float2 *>(s_rgb + NB);
-    float *s_g = reinterpret_cast<float *>(s_ad + NB);
-    unsigned int *s_mask = reinterpret_cast<unsigned int *>(s_g + 9 * NB);
+    float4 *s_g4 = s_dyn + (BS / 32) * RED_VISITS * 32;
+    float2 *s_g2 = reinterpret_cast<float2 *>(s_g4 + BS);
+    float4 *s_st = reinterpret_cast<float4 *>(s_g2 + BS);
+    float *s_g = reinterpret_cast<float *>(s_st + 3 * NB);
+    unsigned char *s_mask = reinterpret_cast<unsigned char *>(s_g + 9 * NB);
     __shared__ int s_item;
-    __shared__ float s_l1[BS / 32];
+    __shared__ Pack s_pack;
+    __shared__ float s_l1[R::WARPS];
     // the projection backward that follows (launched as a programmatic
     // dependent) may start its blocks on SMs this kernel leaves in its tail:
     // it zeroes its gradient rows there, then waits for this grid to finish
     launch_dependents();
     if (counters[CNT_ABORT]) return;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
     const unsigned int wbit = 1u << (threadIdx.x >> 5);
-    // this warp's buffer: row 9 s + j holds value j of the warp's pending
-    // visit s (s < RED_SLOTS), column l that of lane l
-    float *rb = s_red + (threadIdx.x >> 5) * RED_WARP_FLOATS;
-    // at a flush, lane 9 s + j (j < 9) adds row 9 s + j: value j of pending
-    // visit s, whose staged index lane s holds
-    const int red_j = lane % 9, red_s = lane / 9;
-    const float4 *red_row = reinterpret_cast<const float4 *>(rb + lane * RED_PITCH);
-    for (int k = threadIdx.x; k < NB; k += BS)
-        for (int c = 0; c < 9; ++c) s_g[9 * k + c] = 0.f;
+    // this warp's pending visits, and this lane's entry in the next one's row
+    float4 *rb = s_dyn + (threadIdx.x >> 5) * RED_VISITS * 32;
+    const int red0 = red_at(lane);
+    int red_next = red0;
+    for (int k = threadIdx.x; k < 9 * NB; k += BS) s_g[k] = 0.f;
     float l1_sum = 0.f;   // with l1_target: this thread's sum of |image - target|
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(counters + CNT_Q_BWD, 1);
         __syncthreads();
         const int item = s_item;
         __syncthreads();
-        if (item >= L.n_tiles) break;
-        const int tile = order[item];
-        const TileInfo ti = tile_info<TW, TH>(L, tile);
+        if (item >= L.n_tiles * R::PARTS) break;
+        const int tile = order[item / R::PARTS];
+        const TileInfo ti = tile_info<TW, TH>(L, tile, item % R::PARTS);
         const int2 r = ranges[tile];
         const ViewDesc &vd = L.v[ti.view];
         const long long hw = (long long)vd.W * vd.H;
@@ -417,51 +566,34 @@ __global__ void __launch_bounds__(TW * TH / 2, 1024 / (TW * TH / 2)) k_render_bw
         const float2 PCY = make_float2(ti.pcy0, ti.pcy0 + 4.f);
         float2 T = f2(1.f), CG = f2(0.f);
         unsigned int n_eval = 0, n_comp = 0;
+        // the upstream gradients for the sums over visits (read by this warp only)
+        s_g4[warp0 + red0] = make_float4(GR.x, GR.y, GG.x, GG.y);
+        s_g2[warp0 + red0] = GB;
         // the warp's pending visits (warp-uniform) and, in lane s, the staged
         // index of pending visit s
         int npend = 0, kpend = 0;
-        // add the pending visits' rows to their Gaussians' sums in s_g (each
-        // row over the 32 lanes: two f32x2 chains over 8 16-byte loads, then
-        // the two lanes of the pair)
-        auto flush = [&]() {
-            __syncwarp();
-            const int kk = __shfl_sync(0xffffffffu, kpend, red_s);
-            if (lane < 9 * npend) {
-                float4 v = red_row[0];
-                float2 sa = make_float2(v.x, v.y), sb = make_float2(v.z, v.w);
-#pragma unroll
-                for (int i = 1; i < 8; ++i) {
-                    v = red_row[i];
-                    sa = __fadd2_rn(sa, make_float2(v.x, v.y));
-                    sb = __fadd2_rn(sb, make_float2(v.z, v.w));
+        for (int pos = r.x; pos < r.y;) {
+            if (__syncthreads_count(LAST ? pos >= endm : done0 && done1) == BS) break;
+            const int nb = stage_batch<TW, TH>(L, proj, ids, pos, r.y, L.bwd_batch, ti, s_st, s_mask, &s_pack);
+            // the warp takes only the staged Gaussians that may reach its patch, in
+            // order: 32 masks per ballot, then the set bits; the pending visits are
+            // summed when the buffer is full and once at the end of the batch
+            int k0 = -32;
+            unsigned int hits = 0u;
+            for (;;) {
+                bool last = false;
+                while (!hits) {
+                    k0 += 32;
+                    // the end of the batch, or the warp's pixels have all stopped
+                    last = k0 >= nb || __all_sync(0xffffffffu, LAST ? __float_as_int(s_st[3 * k0 + 2].w) >= endm
+                                                                    : done0 && done1);
+                    if (last) break;
+                    hits = __ballot_sync(0xffffffffu, k0 + lane < nb && (s_mask[k0 + lane] & wbit));
                 }
-                sa = __fadd2_rn(sa, sb);
-                atomicAdd(&s_g[9 * kk + red_j], sa.x + sa.y);
-            }
-            npend = 0;
-            __syncwarp();   // the buffer is free for the next visits
-        };
-        for (int b0 = r.x; b0 < r.y; b0 += NB) {
-            if (__syncthreads_count(LAST ? b0 >= endm : done0 && done1) == BS) break;
-            // LAST: the pixels' ends relative to this batch
-            const int e0 = end0 - b0, e1 = end1 - b0;
-            stage_batch<TW, TH>(L, proj, ids, b0, r.y, L.bwd_batch, ti, s_xy, s_con, s_rgb, s_mask);
-            for (int h = 0; h < L.bwd_batch; ++h) {
-                const int k = threadIdx.x + h * BS;
-                if (b0 + k < r.y)
-                    s_ad[k] = make_float2(s_con[k].x * (-2.f * LN2), s_con[k].z * (-2.f * LN2));
-            }
-            __syncthreads();
-            const int nb = min(NB, r.y - b0);
-            for (int k0 = 0; k0 < nb; k0 += 32) {
-                // the warp's pixels have all stopped
-                if (__all_sync(0xffffffffu, LAST ? b0 + k0 >= endm : done0 && done1)) break;
-                // only the staged Gaussians that may reach this warp's patch, in order
-                unsigned int hits = __ballot_sync(0xffffffffu, k0 + lane < nb && (s_mask[k0 + lane] & wbit));
-                while (hits) {
+                if (!last) {
                     const int k = k0 + __ffs(hits) - 1;
                     hits &= hits - 1;
-                    const float4 xy = s_xy[k], con = s_con[k];
+                    const float4 xy = s_st[3 * k], con = s_st[3 * k + 1], c = s_st[3 * k + 2];
                     // both pixels' alphas, the forward's arithmetic and decisions
                     const float dx = __fsub_rn(ti.pcx, xy.x);
                     const bool col = fabsf(dx) <= xy.z;   // the column gate, shared by both pixels
@@ -471,7 +603,8 @@ __global__ void __launch_bounds__(TW * TH / 2, 1024 / (TW * TH / 2)) k_render_bw
                     const float2 G = make_float2(ex2_approx(p2.x), ex2_approx(p2.y));
                     const float2 oG = __fmul2_rn(f2(con.w), G);
                     const float a0 = fminf(oG.x, L.alpha_max), a1 = fminf(oG.y, L.alpha_max);
-                    const bool live0 = LAST ? k < e0 : !done0, live1 = LAST ? k < e1 : !done1;
+                    const int index = __float_as_int(c.w);
+                    const bool live0 = LAST ? index < end0 : !done0, live1 = LAST ? index < end1 : !done1;
                     const bool ev0 = col && live0 && fabsf(dy.x) <= xy.w, ev1 = col && live1 && fabsf(dy.y) <= xy.w;
                     const bool ok0 = ev0 && a0 >= L.alpha_min, ok1 = ev1 && a1 >= L.alpha_min;
                     if (COUNT) n_eval += (unsigned int)ev0 + (unsigned int)ev1;
@@ -502,14 +635,11 @@ __global__ void __launch_bounds__(TW * TH / 2, 1024 / (TW * TH / 2)) k_render_bw
                         Tn = make_float2(cp0 ? Tt.x : T.x, cp1 ? Tt.y : T.y);
                     }
                     if (COUNT) n_comp += (unsigned int)cp0 + (unsigned int)cp1;
-                    // gradients; a pixel that does not composite contributes zeros
-                    // (its weight and its alpha factors are zero)
-                    const float4 c = s_rgb[k];
-                    const float2 ad = s_ad[k];
+                    // a pixel that does not composite contributes zeros (its
+                    // weight and its alpha factor are zero)
                     const float2 w = __fmul2_rn(ac, T);
                     const float2 Told = T;
                     T = Tn;
-                    const float2 g6 = __fmul2_rn(w, GR), g7 = __fmul2_rn(w, GG), g8 = __fmul2_rn(w, GB);
                     // c.g, and C.g accumulated through this Gaussian; S.g = image.g - C.g,
                     // dL/dalpha = T (c.g) - (S.g) / (1 - alpha) (1 - alpha >= 0.01, so
                     // the approximate reciprocal's few-ulp error is far inside the
@@ -519,74 +649,91 @@ __global__ void __launch_bounds__(TW * TH / 2, 1024 / (TW * TH / 2)) k_render_bw
                     const float2 q = __fmul2_rn(__fadd2_rn(CG, NIG), make_float2(rcp_approx(oma.x), rcp_approx(oma.y)));
                     const float2 dla = __ffma2_rn(Told, cgk, q);
                     // alpha = o G unless clamped; G = exp(power), power = -1/2 d^T Q d,
-                    // Q the conic, d = pixel - mean. With v = Q d = (A u, A beta u + D dy)
-                    // from the staged form, d power / d mean = v and d power / d Sigma' =
-                    // v v^T / 2, i.e. (v0^2/2, v0 v1, v1^2/2) for (a, b, c); summing these
-                    // well-scaled terms avoids the ill-conditioned conic -> covariance
-                    // conversion of summed conic gradients. The halves of the (a) and (c)
-                    // sums are applied once, at the flush. Gu = G where the pixel composites
-                    // an unclamped alpha, else 0; d alpha / d power = o Gu.
-                    const bool un0 = cp0 && oG.x <= L.alpha_max, un1 = cp1 && oG.y <= L.alpha_max;
-                    const float2 g5 = __fmul2_rn(dla, make_float2(un0 ? G.x : 0.f, un1 ? G.y : 0.f));
-                    const float2 dp = __fmul2_rn(f2(con.w), g5);
-                    const float2 v0 = __fmul2_rn(f2(ad.x), u);
-                    const float2 v1 = __ffma2_rn(v0, f2(con.y), __fmul2_rn(f2(ad.y), dy));
-                    const float2 g0 = __fmul2_rn(dp, v0), g1 = __fmul2_rn(dp, v1);
-                    const float2 g2 = __fmul2_rn(g0, v0), g3 = __fmul2_rn(g0, v1), g4 = __fmul2_rn(g1, v1);
-                    if (__any_sync(0xffffffffu, cp0 || cp1)) {
-                        // gradient of this thread's pixels w.r.t. (x, y, a, b, c, o, r, g, b),
-                        // as column `lane` of the next pending visit's rows
-                        float *wr = rb + npend * (9 * RED_PITCH) + lane;
-                        wr[0 * RED_PITCH] = g0.x + g0.y;
-                        wr[1 * RED_PITCH] = g1.x + g1.y;
-                        wr[2 * RED_PITCH] = g2.x + g2.y;
-                        wr[3 * RED_PITCH] = g3.x + g3.y;
-                        wr[4 * RED_PITCH] = g4.x + g4.y;
-                        wr[5 * RED_PITCH] = g5.x + g5.y;
-                        wr[6 * RED_PITCH] = g6.x + g6.y;
-                        wr[7 * RED_PITCH] = g7.x + g7.y;
-                        wr[8 * RED_PITCH] = g8.x + g8.y;
-                        kpend = lane == npend ? k : kpend;
-                        if (++npend == RED_SLOTS) flush();
-                    }
+                    // Q the conic, d = pixel - mean: d alpha / d power = alpha where it
+                    // is composited unclamped, else 0. With v = Q d, d power / d mean = v
+                    // and d power / d Sigma' = v v^T / 2, i.e. (v0^2/2, v0 v1, v1^2/2) for
+                    // (a, b, c); summing these well-scaled terms (reduce_visits) avoids
+                    // the ill-conditioned conic -> covariance conversion of summed
+                    // conic gradients.
+                    const float2 dp = __fmul2_rn(dla, make_float2(oG.x <= L.alpha_max ? ac.x : 0.f,
+                                                                  oG.y <= L.alpha_max ? ac.y : 0.f));
+                    if (!LAST && !__any_sync(0xffffffffu, cp0 || cp1)) continue;
+                    rb[red_next] = make_float4(w.x, w.y, dp.x, dp.y);
+                    red_next = (red_next + 32) ^ 4;
+                    kpend = lane == npend ? k : kpend;
+                    if (++npend < RED_VISITS) continue;
+                } else if (npend == 0) {
+                    break;
                 }
+                __syncwarp();
+                reduce_visits(rb, s_g4 + warp0, s_g2 + warp0, npend, __shfl_sync(0xffffffffu, kpend, lane >> 2),
+                              ti.pcx - (float)(lane & 7), ti.pcy0 - (float)(lane >> 3), s_st, s_g);
+                npend = 0;
+                red_next = red0;
+                __syncwarp();   // the buffer is free for the next visits
+                if (last) break;
             }
-            if (npend) flush();   // (warp-uniform) before the batch's sums leave
             __syncthreads();
-            // flush this batch's per-Gaussian sums
+            // the batch's Gaussians that got a sum: the nine gradients, with
+            // A, D the conic's terms in natural-log units and v = (A u, beta A u + D dy)
             for (int h = 0; h < L.bwd_batch; ++h) {
                 const int k = threadIdx.x + h * BS;
                 if (k < nb) {
-                    const float *sg = s_g + 9 * k;
-                    const float a0 = sg[0], a1 = sg[1], a2 = 0.5f * sg[2], a3 = sg[3];
-                    const float a4 = 0.5f * sg[4];
-                    const float a5 = sg[5], a6 = sg[6], a7 = sg[7], a8 = sg[8];
-                    if (a0 != 0.f || a1 != 0.f || a2 != 0.f || a3 != 0.f || a4 != 0.f || a5 != 0.f || a6 != 0.f ||
-                        a7 != 0.f || a8 != 0.f) {
-                        const unsigned int slot = __float_as_uint(s_rgb[k].w);
-                        float4 *dst = grad2d + 3ull * slot;
-                        atomicAdd(dst, make_float4(a0, a1, a2, a3));
-                        atomicAdd(dst + 1, make_float4(a4, a5, a6, a7));
-                        atomicAdd(dst + 2, make_float4(a8, 0.f, 0.f, 0.f));
-                    }
+                    float *sg = s_g + 9 * k;
+                    float t[9];
+                    unsigned int any = 0u;
 #pragma unroll
-                    for (int cc = 0; cc < 9; ++cc) s_g[9 * k + cc] = 0.f;
+                    for (int j = 0; j < 9; ++j) {
+                        t[j] = sg[j];
+                        any |= __float_as_uint(t[j]);
+                    }
+                    if (any & 0x7fffffffu) {
+                        const float4 con = s_st[3 * k + 1];
+                        const float A = con.x * (-2.f * LN2), D = con.z * (-2.f * LN2), beta = con.y;
+                        const float g0 = A * t[1], g1 = fmaf(beta, g0, D * t[2]);
+                        const float g2 = A * A * t[3], ad = A * t[4];                   // sum dp v0^2, sum dp v0 dy
+                        const float g3 = fmaf(beta, g2, D * ad);                        // sum dp v0 v1
+                        const float g4 = fmaf(beta, g3, D * fmaf(beta, ad, D * t[5]));  // sum dp v1^2
+                        float4 *dst = grad2d + 3ull * ids[__float_as_int(s_st[3 * k + 2].w)];
+                        atomicAdd(dst, make_float4(g0, g1, 0.5f * g2, g3));
+                        atomicAdd(dst + 1, make_float4(0.5f * g4, t[0] / con.w, t[6], t[7]));
+                        atomicAdd(dst + 2, make_float4(t[8], 0.f, 0.f, 0.f));
+#pragma unroll
+                        for (int j = 0; j < 9; ++j) sg[j] = 0.f;
+                    }
                 }
             }
         }
         if (COUNT) count_pairs(counters, 12, n_eval, n_comp);
     }
     if (l1_loss) {
-        // the block's part of the loss: one atomic per block (the loss's last
-        // bits depend on their order)
+        // the block's part of the loss
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) l1_sum += __shfl_xor_sync(0xffffffffu, l1_sum, o);
         if (lane == 0) s_l1[threadIdx.x >> 5] = l1_sum;
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (threadIdx.x < 32) {
             float t = 0.f;
-            for (int w = 0; w < BS / 32; ++w) t += s_l1[w];
-            atomicAdd(l1_loss, t * l1_inv_n);
+            for (int w = 0; w < R::WARPS; ++w) t += s_l1[w];
+            if (!l1_part) {
+                if (lane == 0) atomicAdd(l1_loss, t * l1_inv_n);
+                return;
+            }
+            // the last block to get here adds up the parts (a thousand or more
+            // of them: an atomic sum would round each addition to the whole)
+            int done = 0;
+            if (lane == 0) {
+                __stcg(l1_part + blockIdx.x, t);
+                __threadfence();
+                done = atomicAdd(counters + CNT_L1_DONE, 1);
+            }
+            if (__shfl_sync(0xffffffffu, done, 0) != (int)gridDim.x - 1) return;
+            __threadfence();
+            float sum = 0.f;
+            for (int i = lane; i < (int)gridDim.x; i += 32) sum += __ldcg(l1_part + i);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0) *l1_loss = sum * l1_inv_n;
         }
     }
 }
@@ -623,7 +770,7 @@ int launch_zero_accumulators(float *grad2d, long long n_floats, float *loss, cud
 
 // Resident blocks per SM of a raster kernel at the launch's block and
 // dynamic shared-memory size (cached per batch size; the attribute that
-// allows more dynamic shared memory than so far is set on first use).
+// allows more than 48 KB of dynamic shared memory is set on first use).
 template <typename K>
 static int raster_blocks_per_sm(K kernel, int threads, size_t smem, int batch, int *cache) {
     if (!cache[batch]) {
@@ -664,9 +811,10 @@ __device__ __forceinline__ int work_bucket(int w) {
     const int e = 31 - __clz(w);
     return min(1023, e * 32 + ((w >> max(0, e - 5)) & 31));
 }
-__global__ void __launch_bounds__(1024) k_order_by_work(const int *__restrict__ work,
-                                                       const int2 *__restrict__ ranges, int n_tiles,
-                                                       int *__restrict__ order) {
+// With reset, the record is zeroed after it has been read (the forward that
+// follows takes the maximum over a tile's pixels into it).
+__global__ void __launch_bounds__(1024) k_order_by_work(int *__restrict__ work, const int2 *__restrict__ ranges,
+                                                        int n_tiles, int *__restrict__ order, bool reset) {
     __shared__ int s_cnt[1024];
     __shared__ int s_part[32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -704,16 +852,20 @@ __global__ void __launch_bounds__(1024) k_order_by_work(const int *__restrict__ 
     __syncthreads();
     s_cnt[1023 - tid] = s_part[wid] + incl - c;   // the bucket's first position
     __syncthreads();
-    for (int t = tid; t < n_tiles; t += 1024) order[atomicAdd(&s_cnt[work_bucket(predicted(t))], 1)] = t;
+    for (int t = tid; t < n_tiles; t += 1024) {
+        order[atomicAdd(&s_cnt[work_bucket(predicted(t))], 1)] = t;
+        if (reset) work[t] = 0;
+    }
 }
 
 template <int TW, int TH>
 static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, float *image, cudaStream_t st) {
+    using R = Region<TW, TH>;
     static int blocks_per_sm[5];
-    const size_t smem = (size_t)FWD_STAGE_BYTES * L.fwd_batch * (TW * TH / 2);
-    const int grid = min(num_sms() * raster_blocks_per_sm(k_render_fwd<TW, TH>, TW * TH / 2, smem, L.fwd_batch,
-                                                          blocks_per_sm),
-                         max(1, L.n_tiles));
+    const size_t smem = (size_t)FWD_STAGE_BYTES * L.fwd_batch * R::BS;
+    const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_fwd<TW, TH>, R::BS, smem,
+                                                                          L.fwd_batch, blocks_per_sm),
+                              max(1LL, (long long)L.n_tiles * R::PARTS));
     // every call walks all tiles again: reset this kernel's work-queue head
     if (cudaMemsetAsync(b->counters + CNT_Q_FWD, 0, sizeof(int), st) != cudaSuccess) return GS_ERR_CUDA;
     // with the last-contrib record and few tiles per SM, also each tile's
@@ -724,30 +876,43 @@ static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, fl
     const bool ordered = order_by_work(L, b);
     if (ordered && b->tile_work) {
         k_order_by_work<<<1, 1024, 0, st>>>(b->tile_work, reinterpret_cast<const int2 *>(b->tile_ranges),
-                                            (int)L.n_tiles, b->tile_order);
+                                            (int)L.n_tiles, b->tile_order, true);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
+    } else if (ordered) {
+        if (cudaMemsetAsync(b->tile_scratch, 0, sizeof(int) * (size_t)L.n_tiles, st) != cudaSuccess)
+            return GS_ERR_CUDA;
     }
-    k_render_fwd<TW, TH><<<grid, TW * TH / 2, smem, st>>>(L, reinterpret_cast<const float4 *>(proj),
-                                                       reinterpret_cast<const int2 *>(b->tile_ranges), b->ids,
-                                                       b->tile_order, b->counters, image, b->last_contrib,
-                                                       ordered ? work_record(b) : nullptr);
+    k_render_fwd<TW, TH><<<grid, R::BS, smem, st>>>(L, reinterpret_cast<const float4 *>(proj),
+                                                    reinterpret_cast<const int2 *>(b->tile_ranges), b->ids,
+                                                    b->tile_order, b->counters, image, b->last_contrib,
+                                                    ordered ? work_record(b) : nullptr);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 template <int TW, int TH, bool COUNT, bool LAST>
 static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, const float *image,
                         const float *dL_dimage, const L1Loss &l1, float *grad2d, cudaStream_t st) {
+    using R = Region<TW, TH>;
     static int blocks_per_sm[5];
-    const size_t smem = (size_t)BWD_STAGE_BYTES * L.bwd_batch * (TW * TH / 2) +
-                        sizeof(float) * RED_WARP_FLOATS * (TW * TH / 64);
-    const int grid = min(num_sms() * raster_blocks_per_sm(k_render_bwd<TW, TH, COUNT, LAST>, TW * TH / 2, smem,
-                                                          L.bwd_batch, blocks_per_sm),
-                         max(1, L.n_tiles));
-    if (cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, sizeof(int), st) != cudaSuccess) return GS_ERR_CUDA;
-    k_render_bwd<TW, TH, COUNT, LAST><<<grid, TW * TH / 2, smem, st>>>(
+    const size_t smem = (size_t)BWD_STAGE_BYTES * L.bwd_batch * R::BS + (size_t)RED_WARP_BYTES * R::WARPS;
+    const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_bwd<TW, TH, COUNT, LAST>, R::BS,
+                                                                          smem, L.bwd_batch, blocks_per_sm),
+                              max(1LL, (long long)L.n_tiles * R::PARTS));
+    // the queue head, and the count of blocks that have added to the loss
+    static_assert(CNT_L1_DONE == CNT_Q_BWD + 1, "reset together");
+    if (cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, 2 * sizeof(int), st) != cudaSuccess) return GS_ERR_CUDA;
+    // the blocks' parts of the loss lie behind the work record (tile_scratch is
+    // 5 ints per tile; the grid has at most PARTS <= 4 blocks per tile)
+    static_assert(R::PARTS <= 4, "one part of the loss per block fits tile_scratch");
+    // (the ordered sum costs a small launch about 2 us: only where the blocks
+    // are many, or more of them than one per tile)
+    const bool many = grid > (R::PARTS > 1 ? 2 : 8) * num_sms();
+    float *l1_part = l1.loss && b->tile_scratch && many
+                         ? reinterpret_cast<float *>(b->tile_scratch + L.n_tiles) : nullptr;
+    k_render_bwd<TW, TH, COUNT, LAST><<<grid, R::BS, smem, st>>>(
         L, reinterpret_cast<const float4 *>(proj), reinterpret_cast<const int2 *>(b->tile_ranges), b->ids,
         b->tile_order, b->counters, image, dL_dimage, b->last_contrib, reinterpret_cast<float4 *>(grad2d), l1.target,
-        l1.loss, l1.inv_n);
+        l1.loss, l1.inv_n, l1_part);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
@@ -757,7 +922,7 @@ static int launch_bwd_t(const Launch &L, const float *proj, const gs_bins *b, co
     if (b->last_contrib) {
         // the forward recorded each tile's replay length
         if (order_by_work(L, b)) {
-            k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order);
+            k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false);
             if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
         }
         return L.count_pairs ? launch_bwd_c<TW, TH, true, true>(L, proj, b, image, dL_dimage, l1, grad2d, st)
