@@ -284,6 +284,18 @@ __device__ __forceinline__ int stage_batch(const Launch &L, const float4 *__rest
     }
 }
 
+// A persistent block's next item: its first is its own number, the rest come
+// from the queue (none when there is a block per item: such a launch uses no
+// queue). Whole block.
+__device__ __forceinline__ int next_item(int *queue, int items, int *s_item) {
+    if ((int)gridDim.x >= items) return items;
+    if (threadIdx.x == 0) *s_item = (int)gridDim.x + atomicAdd(queue, 1);
+    __syncthreads();
+    const int item = *s_item;
+    __syncthreads();
+    return item;
+}
+
 // Shared-memory bytes of one staged Gaussian: position, conic and colour
 // (3 x 16 B) and the warp mask (a byte: at most four warps); the backward adds
 // its nine sums.
@@ -384,13 +396,11 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, 1024 / Region<TW, TH>::BS)
     const bool abort = counters[CNT_ABORT] != 0;
     const unsigned int wbit = 1u << (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(counters + CNT_Q_FWD, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= L.n_tiles * R::PARTS) break;
+    const int items = L.n_tiles * R::PARTS;
+    for (int item = blockIdx.x; item < items; item = next_item(counters + CNT_Q_FWD, items, &s_item)) {
         const int tile = order[item / R::PARTS];
+        // (a tile of one part: no other block adds to its record)
+        if (R::PARTS == 1 && tile_work && threadIdx.x == 0) tile_work[tile] = 0;
         const TileInfo ti = tile_info<TW, TH>(L, tile, item % R::PARTS);
         const int2 r = abort ? make_int2(0, 0) : ranges[tile];
         // lane .x = pixel (px, py0), lane .y = pixel (px, py0 + 4)
@@ -514,12 +524,9 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>:
     int red_next = red0;
     for (int k = threadIdx.x; k < 9 * NB; k += BS) s_g[k] = 0.f;
     float l1_sum = 0.f;   // with l1_target: this thread's sum of |image - target|
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(counters + CNT_Q_BWD, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= L.n_tiles * R::PARTS) break;
+    const int items = L.n_tiles * R::PARTS;
+    __syncthreads();   // the sums are zero
+    for (int item = blockIdx.x; item < items; item = next_item(counters + CNT_Q_BWD, items, &s_item)) {
         const int tile = order[item / R::PARTS];
         const TileInfo ti = tile_info<TW, TH>(L, tile, item % R::PARTS);
         const int2 r = ranges[tile];
@@ -794,6 +801,11 @@ static int raster_blocks_per_sm(K kernel, int threads, size_t smem, int batch, i
 static bool order_by_work(const Launch &L, const gs_bins *b) {
     return b->last_contrib && L.n_tiles > 0 && L.n_tiles < 16LL * num_sms();
 }
+// Few regions: every one gets a resident block of its own at once (each raster
+// kernel keeps at least four blocks per SM), so neither an order nor a queue
+// matters, and the launches that prepare them are left out (4 to 5 us each in a
+// step of 120 us).
+static bool all_at_once(long long items) { return items <= 4LL * num_sms(); }
 // where the forward records the replay lengths: the caller's kept record,
 // else tile_scratch (this call only)
 static int *work_record(const gs_bins *b) { return b->tile_work ? b->tile_work : b->tile_scratch; }
@@ -812,9 +824,10 @@ __device__ __forceinline__ int work_bucket(int w) {
     return min(1023, e * 32 + ((w >> max(0, e - 5)) & 31));
 }
 // With reset, the record is zeroed after it has been read (the forward that
-// follows takes the maximum over a tile's pixels into it).
+// follows takes the maximum over a tile's pixels into it). The kernel's queue
+// head and the word after it are cleared too.
 __global__ void __launch_bounds__(1024) k_order_by_work(int *__restrict__ work, const int2 *__restrict__ ranges,
-                                                        int n_tiles, int *__restrict__ order, bool reset) {
+                                                        int n_tiles, int *__restrict__ order, bool reset, int *queue) {
     __shared__ int s_cnt[1024];
     __shared__ int s_part[32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -825,6 +838,7 @@ __global__ void __launch_bounds__(1024) k_order_by_work(int *__restrict__ work, 
         return r.y - r.x;
     };
     s_cnt[tid] = 0;
+    if (tid < 2) queue[tid] = 0;
     __syncthreads();
     for (int t = tid; t < n_tiles; t += 1024) atomicAdd(&s_cnt[work_bucket(predicted(t))], 1);
     __syncthreads();
@@ -866,20 +880,23 @@ static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, fl
     const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_fwd<TW, TH>, R::BS, smem,
                                                                           L.fwd_batch, blocks_per_sm),
                               max(1LL, (long long)L.n_tiles * R::PARTS));
-    // every call walks all tiles again: reset this kernel's work-queue head
-    if (cudaMemsetAsync(b->counters + CNT_Q_FWD, 0, sizeof(int), st) != cudaSuccess) return GS_ERR_CUDA;
     // with the last-contrib record and few tiles per SM, also each tile's
     // replay length for the backward's work order: into the kept work record
     // (after taking this forward's order from the previous one's lengths,
     // the instance count where none is recorded; the sort no longer needs
-    // tile_order), else into tile_scratch (free after the sort)
+    // tile_order), else into tile_scratch (free after the sort). A tile of
+    // several parts collects the largest of their lengths, from zero.
+    const long long items = (long long)L.n_tiles * R::PARTS;
     const bool ordered = order_by_work(L, b);
-    if (ordered && b->tile_work) {
+    if (ordered && b->tile_work && !all_at_once(items)) {
         k_order_by_work<<<1, 1024, 0, st>>>(b->tile_work, reinterpret_cast<const int2 *>(b->tile_ranges),
-                                            (int)L.n_tiles, b->tile_order, true);
+                                            (int)L.n_tiles, b->tile_order, true, b->counters + CNT_Q_FWD);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-    } else if (ordered) {
-        if (cudaMemsetAsync(b->tile_scratch, 0, sizeof(int) * (size_t)L.n_tiles, st) != cudaSuccess)
+    } else {
+        // every call walks all tiles again: reset this kernel's work-queue head
+        if (grid < items && cudaMemsetAsync(b->counters + CNT_Q_FWD, 0, sizeof(int), st) != cudaSuccess) return GS_ERR_CUDA;
+        if (ordered && R::PARTS > 1 &&
+            cudaMemsetAsync(work_record(b), 0, sizeof(int) * (size_t)L.n_tiles, st) != cudaSuccess)
             return GS_ERR_CUDA;
     }
     k_render_fwd<TW, TH><<<grid, R::BS, smem, st>>>(L, reinterpret_cast<const float4 *>(proj),
@@ -891,7 +908,7 @@ static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, fl
 
 template <int TW, int TH, bool COUNT, bool LAST>
 static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, const float *image,
-                        const float *dL_dimage, const L1Loss &l1, float *grad2d, cudaStream_t st) {
+                        const float *dL_dimage, const L1Loss &l1, float *grad2d, bool queue_reset, cudaStream_t st) {
     using R = Region<TW, TH>;
     static int blocks_per_sm[5];
     const size_t smem = (size_t)BWD_STAGE_BYTES * L.bwd_batch * R::BS + (size_t)RED_WARP_BYTES * R::WARPS;
@@ -900,13 +917,15 @@ static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, co
                               max(1LL, (long long)L.n_tiles * R::PARTS));
     // the queue head, and the count of blocks that have added to the loss
     static_assert(CNT_L1_DONE == CNT_Q_BWD + 1, "reset together");
-    if (cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, 2 * sizeof(int), st) != cudaSuccess) return GS_ERR_CUDA;
+    if (!queue_reset && grid < (long long)L.n_tiles * R::PARTS &&
+        cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, 2 * sizeof(int), st) != cudaSuccess)
+        return GS_ERR_CUDA;
     // the blocks' parts of the loss lie behind the work record (tile_scratch is
     // 5 ints per tile; the grid has at most PARTS <= 4 blocks per tile)
     static_assert(R::PARTS <= 4, "one part of the loss per block fits tile_scratch");
     // (the ordered sum costs a small launch about 2 us: only where the blocks
     // are many, or more of them than one per tile)
-    const bool many = grid > (R::PARTS > 1 ? 2 : 8) * num_sms();
+    const bool many = grid > (R::PARTS > 1 ? 4 : 8) * num_sms();
     float *l1_part = l1.loss && b->tile_scratch && many
                          ? reinterpret_cast<float *>(b->tile_scratch + L.n_tiles) : nullptr;
     k_render_bwd<TW, TH, COUNT, LAST><<<grid, R::BS, smem, st>>>(
@@ -921,15 +940,17 @@ static int launch_bwd_t(const Launch &L, const float *proj, const gs_bins *b, co
                         const float *dL_dimage, const L1Loss &l1, float *grad2d, cudaStream_t st) {
     if (b->last_contrib) {
         // the forward recorded each tile's replay length
-        if (order_by_work(L, b)) {
-            k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false);
+        const bool ordered = order_by_work(L, b) && !all_at_once((long long)L.n_tiles * Region<TW, TH>::PARTS);
+        if (ordered) {
+            k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false,
+                                                b->counters + CNT_Q_BWD);
             if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
         }
-        return L.count_pairs ? launch_bwd_c<TW, TH, true, true>(L, proj, b, image, dL_dimage, l1, grad2d, st)
-                             : launch_bwd_c<TW, TH, false, true>(L, proj, b, image, dL_dimage, l1, grad2d, st);
+        return L.count_pairs ? launch_bwd_c<TW, TH, true, true>(L, proj, b, image, dL_dimage, l1, grad2d, ordered, st)
+                             : launch_bwd_c<TW, TH, false, true>(L, proj, b, image, dL_dimage, l1, grad2d, ordered, st);
     }
-    return L.count_pairs ? launch_bwd_c<TW, TH, true, false>(L, proj, b, image, dL_dimage, l1, grad2d, st)
-                         : launch_bwd_c<TW, TH, false, false>(L, proj, b, image, dL_dimage, l1, grad2d, st);
+    return L.count_pairs ? launch_bwd_c<TW, TH, true, false>(L, proj, b, image, dL_dimage, l1, grad2d, false, st)
+                         : launch_bwd_c<TW, TH, false, false>(L, proj, b, image, dL_dimage, l1, grad2d, false, st);
 }
 
 int launch_render_fwd(const Launch &L, const float *proj, const gs_bins *b, float *image, cudaStream_t st) {

@@ -40,11 +40,12 @@ from .autograd import Rasterizer
 
 
 class GraphStep:
-    # project 1, bin/sort 5 (count, scan, scatter, split, sort), render 1, the
-    # zeroing of the backward's accumulators 1 (a kernel with overlap_prev),
-    # raster bwd 1, projection bwd 1, pose 1; the L1 loss is part of the raster
-    # backward, the L1 + D-SSIM loss adds 1 kernel
-    KERNELS_FIXED = 11
+    # project 1, bin/sort 4 (count, scan, scatter, sort), render 1, the zeroing of
+    # the backward's accumulators 1 (a kernel with overlap_prev), raster bwd 1,
+    # projection bwd 1, pose 1; the L1 loss is part of the raster backward, the
+    # L1 + D-SSIM loss adds 1 kernel
+    KERNELS_FIXED = 10
+    SORT_CAP = 4096   # tiles above it may be split (one more kernel where a view has that many Gaussians)
     # the calls of a step, in order (the stages of run()'s events)
     STAGES = {"l1": ("gs_project", "gs_bin_sort", "gs_render_fwd", "gs_rasterize_bwd_l1", "gs_project_bwd",
                      "gs_pose_grad"),
@@ -56,14 +57,19 @@ class GraphStep:
         return self.STAGES[self.loss_kind]
 
     def kernels_per_step(self) -> int:
-        """Kernels of this library that one step launches: the fixed eleven, the
-        D-SSIM loss kernel, and, when the image has fewer than 16 tiles per
-        SM, the tile orderings by replay length that the raster forward (from
-        the previous forward's record) and the raster backward run first."""
+        """Kernels of this library that one step launches: the fixed ten, the
+        D-SSIM loss kernel, the split of large tiles where a view has Gaussians
+        enough for one, and, when the image has fewer than 16 tiles per SM but
+        more regions than get a block at once (four per SM), the tile orderings
+        by replay length that the raster forward (from the previous forward's
+        record) and the raster backward run first."""
         loss = 0 if self.loss_kind == "l1" else 1
         sms = torch.cuda.get_device_properties(self.g.means.device).multi_processor_count
-        order = 2 if 0 < self.bins.n_tiles < 16 * sms else 0
-        return self.KERNELS_FIXED + loss + order
+        area = self.cfg.tile_w * self.cfg.tile_h
+        regions = self.bins.n_tiles * (area // 256 if area > 256 else 1)
+        order = 2 if 0 < self.bins.n_tiles < 16 * sms and regions > 4 * sms else 0
+        split = 1 if int(self.views.gauss_count.max()) > self.SORT_CAP else 0
+        return self.KERNELS_FIXED + loss + order + split
 
     def __init__(self, g: Gaussians, views: Views, target, tile=(16, 16), headroom=1.25, capture=True,
                  want_gaussian_grads=True, loss="l1", lam=0.2, slots=1, slot_gaussians=False, capacity=None,
