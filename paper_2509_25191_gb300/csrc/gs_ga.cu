@@ -649,14 +649,16 @@ __global__ void __launch_bounds__(GA_SEL_THREADS) k_ga_inc_sort(const int32_t *_
 // that share the lower median's top bits; (c) the weights and the last 11 bits.
 // The last block of each pass to finish picks the pass's digit of the lower
 // median (and in (b) forms the table of weights), so no launch lies between the
-// passes. The upper median is the next key: in the same final histogram, or the
-// smallest key above its range, which (c) keeps as a minimum.
+// passes. The upper median is the next key: in the same final histogram (searched by
+// the whole block: one thread's walk over its bins took 80 us where few distances
+// leave it sparse), or the smallest key above its range, which (c) keeps as a minimum.
 // Bound: 4 B read per pass and 4 B written (HBM for the first pass, mostly L2
-// after it where the distances fit). 21.3M distances: 92 us, against 285 us for
-// nine passes with six one-warp digit picks between them; counters in one copy per block
-// alone took 46 us for the bin counts, since most distances fall into the first
-// few bins and the lanes of a warp then queue for one address. Here neighbouring
-// lanes count in different copies (up to 32) of the counters.
+// after it where the distances fit). 21.3M distances: 92 us, 70,574: 32 us, against
+// 285 and 93 us for nine passes with six one-warp digit picks between them;
+// counters in one copy per block alone took 46 us for the bin counts, since most
+// distances fall into the first few bins and the lanes of a warp then queue for
+// one address. Here neighbouring lanes count in different copies (up to 32) of
+// the counters.
 // scratch words: [0] max bits, [1] prefix of the lower median's key, [2] its rank
 // among the keys with that prefix, [3..5] blocks done per pass, [6] smallest key
 // above the prefix's range (complemented), [8..8+2048) digit histogram,
@@ -666,7 +668,8 @@ constexpr int GA_W_HIST = 8;
 constexpr int GA_W_TABLE = 8 + GA_RADIX_BINS;
 constexpr int GA_W_THREADS = 512;
 constexpr int GA_W_B0 = 10, GA_W_B1 = 11, GA_W_B2 = 11;   // bits of the key's digits from the top
-constexpr int GA_W_COPY_WORDS = 16384;       // shared words for the copies of a pass's first counters
+constexpr int GA_W_COPY_WORDS = 10240;       // shared words for the copies of a pass's first counters: a pass
+                                             // stays within 48 KB but for more than 10,240 bins
 static_assert(GA_W_B0 + GA_W_B1 + GA_W_B2 == 32 && (1 << GA_W_B1) <= GA_RADIX_BINS, "key digits");
 
 // copies of nb counters (a power of two, at most 32) that fit the shared words
@@ -715,11 +718,12 @@ __device__ __forceinline__ bool ga_last_block(uint32_t *done) {
 // The digit of the histogram (2^bits bins, bits 10 or 11) that holds the rank:
 // scratch[1] |= digit << shift, scratch[2] becomes the rank within the digit, the
 // histogram is cleared. Whole block; returns the digit, and in *count the number
-// of keys in it.
+// of keys in it and in *next the next digit that has a key (2^bits if none).
 template <int BITS>
-__device__ __forceinline__ uint32_t ga_pick(uint32_t *scratch, uint32_t rank, int shift, uint32_t *count) {
+__device__ __forceinline__ uint32_t ga_pick(uint32_t *scratch, uint32_t rank, int shift, uint32_t *count,
+                                            uint32_t *next) {
     constexpr int PER = (1 << BITS) / GA_W_THREADS;
-    __shared__ uint32_t s_part[GA_W_THREADS / 32], s_digit, s_count;
+    __shared__ uint32_t s_part[GA_W_THREADS / 32], s_digit, s_count, s_next;
     uint32_t *h = scratch + GA_W_HIST;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t c[PER], local = 0;
@@ -735,6 +739,7 @@ __device__ __forceinline__ uint32_t ga_pick(uint32_t *scratch, uint32_t rank, in
         if (lane >= o) incl += v;
     }
     if (lane == 31) s_part[wid] = incl;
+    if (threadIdx.x == 0) s_next = 1u << BITS;
     __syncthreads();
     for (int w = 0; w < wid; ++w) incl += s_part[w];
     uint32_t at = incl - local;
@@ -752,6 +757,17 @@ __device__ __forceinline__ uint32_t ga_pick(uint32_t *scratch, uint32_t rank, in
     }
     __syncthreads();
     if (count) *count = s_count;
+    if (next) {
+        uint32_t mine = 1u << BITS;
+#pragma unroll
+        for (int k = PER - 1; k >= 0; --k) {
+            const uint32_t d = (uint32_t)(threadIdx.x * PER + k);
+            if (c[k] && d > s_digit) mine = d;   // (ends at the thread's smallest)
+        }
+        if (mine < (1u << BITS)) atomicMin(&s_next, mine);
+        __syncthreads();
+        *next = s_next;
+    }
     return s_digit;
 }
 
@@ -783,7 +799,7 @@ __global__ void __launch_bounds__(GA_W_THREADS) k_ga_w_max(const float *__restri
         if (c) atomicAdd(&scratch[GA_W_HIST + b], c);
     }
     if (!ga_last_block(scratch + 3)) return;
-    ga_pick<GA_W_B0>(scratch, rank, SH, nullptr);
+    ga_pick<GA_W_B0>(scratch, rank, SH, nullptr, nullptr);
     ga_clear_hist<GA_W_B0>(scratch);
 }
 
@@ -840,7 +856,7 @@ __global__ void __launch_bounds__(GA_W_THREADS) k_ga_w_count(const float *__rest
         if (s_d[b]) atomicAdd(&scratch[GA_W_HIST + b], s_d[b]);
     if (!ga_last_block(scratch + 4)) return;
     ga_table(counts, nb, n, alpha, scratch);
-    ga_pick<GA_W_B1>(scratch, scratch[2], SH, nullptr);
+    ga_pick<GA_W_B1>(scratch, scratch[2], SH, nullptr, nullptr);
     ga_clear_hist<GA_W_B1>(scratch);
 }
 
@@ -881,16 +897,14 @@ __global__ void __launch_bounds__(GA_W_THREADS) k_ga_w_gather(const float *__res
     for (int b = threadIdx.x; b < DIG; b += GA_W_THREADS)
         if (s_h[b]) atomicAdd(&scratch[GA_W_HIST + b], s_h[b]);
     if (!ga_last_block(scratch + 5)) return;
-    uint32_t in_digit;
-    const uint32_t digit = ga_pick<GA_W_B2>(scratch, scratch[2], 0, &in_digit);
+    uint32_t in_digit, next;
+    ga_pick<GA_W_B2>(scratch, scratch[2], 0, &in_digit, &next);
     if (threadIdx.x == 0) {
         const uint32_t lo = scratch[1];
         uint32_t hi = lo;
         if ((n & 1) == 0 && scratch[2] + 1u >= in_digit) {
             // the next key: the next bin of this histogram, or the smallest above
-            uint32_t d = digit + 1;
-            while (d < DIG && __ldcg(scratch + GA_W_HIST + d) == 0u) ++d;
-            hi = d < DIG ? (top << GA_W_B2) | d : ~__ldcg(scratch + 6);
+            hi = next < (uint32_t)DIG ? (top << GA_W_B2) | next : ~__ldcg(scratch + 6);
         }
         stats[0] = emax;
         stats[1] = __uint_as_float(lo);
@@ -988,12 +1002,12 @@ int launch_ga_weights(const float *e, long long n, int nb, double alpha, uint32_
     const int c0 = ga_copies(1 << GA_W_B0), c1 = ga_copies(nb);
     const size_t m0 = 4ull * c0 << GA_W_B0, m1 = 4ull * ((size_t)c1 * nb + (1 << GA_W_B1)),
                  m2 = 4ull * ((1 << GA_W_B2) + (size_t)nb);
-    // (the largest each kernel is ever launched with: the same setting from every call)
-    const int most = 4 * (GA_W_COPY_WORDS + GA_RADIX_BINS);
-    static_assert(GS_GA_MAX_BINS <= GA_W_COPY_WORDS, "one copy of the bin counters fits");
-    if (cudaFuncSetAttribute(k_ga_w_max, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
-        cudaFuncSetAttribute(k_ga_w_count, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
-        cudaFuncSetAttribute(k_ga_w_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess)
+    // (set only where it is needed: the call costs more than a small pass)
+    if (m1 > 48 * 1024 &&
+        cudaFuncSetAttribute(k_ga_w_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m1) != cudaSuccess)
+        return GS_ERR_CUDA;
+    if (m2 > 48 * 1024 &&
+        cudaFuncSetAttribute(k_ga_w_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m2) != cudaSuccess)
         return GS_ERR_CUDA;
     // the lower median's rank; the upper one is the next key if n is even
     k_ga_w_max<<<grid, GA_W_THREADS, m0, st>>>(e, n, c0, (uint32_t)((n - 1) / 2), scratch);

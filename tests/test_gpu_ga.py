@@ -338,3 +338,17 @@ def test_weights_three_passes_at_their_edges(n, n_bins, kind):
     lo, hi, _ = OG.median_order_stats(e)
     st = stats.cpu().numpy()
     assert st[0] == e.max() and st[1] == np.float32(lo) and st[2] == np.float32(hi) and st[3] == 0
+
+
+@pytest.mark.parametrize("distance", [1, 2, 700, 2040, 2047, 5000])
+def test_weights_upper_median_far_from_the_lower_one(distance):
+    """An even count whose two middle keys lie a given number of floats apart:
+    the next bin, the last bin of the histogram, and beyond it."""
+    one = int(np.float32(1.0).view(np.uint32))   # (a multiple of the last digit's 2,048 keys)
+    e = np.concatenate([np.full(500, 1.0, np.float32),
+                        np.full(500, one + distance, np.uint32).view(np.float32)])
+    np.random.default_rng(distance).shuffle(e)
+    _, _, stats = ga.pdf_weights(torch.as_tensor(e).cuda(), 100, 0.5)
+    torch.cuda.synchronize()
+    st = stats.cpu().numpy()
+    assert st[1] == np.float32(1.0) and st[2:3].view(np.uint32)[0] == one + distance
