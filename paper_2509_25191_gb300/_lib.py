@@ -139,8 +139,14 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # (the raw handle: a Stream object costs more than the rest of a call's marshalling)
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
+
+
+def _host(a):
+    """Address of a contiguous host array (ndarray.ctypes builds several objects for it)."""
+    return a.__array_interface__["data"][0]
 
 
 # ---------------------------------------------------------------------------
@@ -201,10 +207,8 @@ class Views:
         assert 1 <= self.n <= GS_MAX_VIEWS
 
     def c(self) -> gs_views:
-        return gs_views(self.n, _ptr(self.viewmats), _ptr(self.intrinsics),
-                        self.width.ctypes.data_as(ctypes.c_void_p), self.height.ctypes.data_as(ctypes.c_void_p),
-                        self.gauss_begin.ctypes.data_as(ctypes.c_void_p),
-                        self.gauss_count.ctypes.data_as(ctypes.c_void_p))
+        return gs_views(self.n, _ptr(self.viewmats), _ptr(self.intrinsics), _host(self.width), _host(self.height),
+                        _host(self.gauss_begin), _host(self.gauss_count))
 
     @staticmethod
     def from_synth(views, device="cuda", viewmats=None):
@@ -266,9 +270,10 @@ class Bins:
 
 
 class Grads:
-    """Gradient outputs and backward scratch (device)."""
+    """Gradient outputs and backward scratch (device). With ``scratch`` (another
+    Grads of the same sizes) only the outputs are new."""
 
-    def __init__(self, n, sh_degree, n_slots, n_views, device="cuda", want_gaussian_grads=True):
+    def __init__(self, n, sh_degree, n_slots, n_views, device="cuda", want_gaussian_grads=True, scratch=None):
         K = (sh_degree + 1) ** 2
         f = dict(dtype=torch.float32, device=device)
         nn = max(1, n) if want_gaussian_grads else 1
@@ -277,6 +282,9 @@ class Grads:
         self.quats = torch.empty(nn, 4, **f)
         self.opacity_logits = torch.empty(nn, **f)
         self.sh = torch.empty(nn, K, 3, **f)
+        if scratch is not None:
+            self.grad2d, self.n_blocks, self.pose_partials = scratch.grad2d, scratch.n_blocks, scratch.pose_partials
+            return
         self.grad2d = torch.empty(max(1, n_slots), GS_GRAD2D_FLOATS, **f)
         self.n_blocks = int(load().gs_pose_blocks(ctypes.c_int64(n)))
         self.pose_partials = torch.empty(n_views * self.n_blocks * 12, **f)

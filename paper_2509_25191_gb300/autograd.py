@@ -2,8 +2,8 @@
 
 ``Rasterizer`` owns the device buffers of one views layout (projected
 records, tile lists, gradient scratch) and plans the tile-instance capacity:
-uncaptured calls read the instance count back once per forward (4 bytes) and
-grow the buffers when needed; captured (CUDA graph) calls run with a fixed
+uncaptured calls read the instance count back once per forward (4 bytes, while
+the raster kernel runs) and grow the buffers when needed; captured (CUDA graph) calls run with a fixed
 capacity and report overflow through the device status word.
 
 ``RasterizeViews`` is the autograd.Function: forward = gs_project +
@@ -38,6 +38,7 @@ class Rasterizer:
         self.status = None
         self.fixed_capacity = False   # set for graph capture: never read back
         self._grads = None
+        self._count = None            # pinned host word and event of the count's readback
         self.last_instances = None
         self.generation = 0           # counts bin_sort calls: which forward the tile lists belong to
 
@@ -64,7 +65,7 @@ class Rasterizer:
         _lib.gs_project(g, views, self.cfg, proj, self.status)
         return proj
 
-    def bin_sort(self, views: Views, proj):
+    def _enqueue_bin_sort(self, views: Views, proj):
         dev = proj.device
         if self.bins is None:
             self._ensure_bins(views, max(1024, 4 * views.num_slots()), dev)
@@ -72,18 +73,27 @@ class Rasterizer:
             self._ensure_bins(views, self.bins.capacity, dev)
         _lib.gs_bin_sort(views, self.cfg, proj, self.bins, self.status)
         self.generation += 1
+
+    def _fit(self, views: Views, proj, n: int) -> bool:
+        """After the readback of the instance count n: if the lists were too
+        small, grow them and bin again (True)."""
+        self.last_instances = n
+        if n >= INSTANCE_LIMIT:
+            # the count saturates at 2^31 - 1: more instances than the
+            # 32-bit tile ranges can address; growing cannot help
+            raise _lib.GsError(_lib.GS_ERR_OVERFLOW, f"gs_bin_sort ({n} or more tile instances)")
+        if n <= self.bins.capacity:
+            return False
+        self.status.zero_()
+        self._ensure_bins(views, int(math.ceil(n * self.headroom)) + 1024, proj.device)
+        _lib.gs_bin_sort(views, self.cfg, proj, self.bins, self.status)
+        self.check_status()   # the re-bin must fit (it reads the status word once)
+        return True
+
+    def bin_sort(self, views: Views, proj):
+        self._enqueue_bin_sort(views, proj)
         if not self.fixed_capacity:
-            n = int(self.bins.counters[0].item())   # the one readback of the uncaptured path
-            self.last_instances = n
-            if n >= INSTANCE_LIMIT:
-                # the count saturates at 2^31 - 1: more instances than the
-                # 32-bit tile ranges can address; growing cannot help
-                raise _lib.GsError(_lib.GS_ERR_OVERFLOW, f"gs_bin_sort ({n} or more tile instances)")
-            if n > self.bins.capacity:
-                self.status.zero_()
-                self._ensure_bins(views, int(math.ceil(n * self.headroom)) + 1024, dev)
-                _lib.gs_bin_sort(views, self.cfg, proj, self.bins, self.status)
-                self.check_status()   # the re-bin must fit (it reads the status word once)
+            self._fit(views, proj, int(self.bins.counters[0].item()))   # the one readback of the uncaptured path
         return self.bins
 
     def render(self, views: Views, proj, bins: Bins, image=None):
@@ -94,8 +104,20 @@ class Rasterizer:
 
     def forward(self, g: Gaussians, views: Views):
         proj = self.project(g, views)
-        bins = self.bin_sort(views, proj)
-        image = self.render(views, proj, bins)
+        if self.fixed_capacity:
+            return self.render(views, proj, self.bin_sort(views, proj)), proj
+        # the count is read back while the raster kernel runs (with lists that
+        # turn out too small it writes zeros, and runs again on the new ones)
+        self._enqueue_bin_sort(views, proj)
+        if self._count is None:
+            self._count = torch.empty(1, dtype=torch.int32, pin_memory=True), torch.cuda.Event()
+        count, ready = self._count
+        count.copy_(self.bins.counters[:1], non_blocking=True)
+        ready.record()
+        image = self.render(views, proj, self.bins)
+        ready.synchronize()
+        if self._fit(views, proj, int(count[0])):
+            self.render(views, proj, self.bins, image)
         return image, proj
 
     def grads_buffers(self, g: Gaussians, views: Views, want_gaussian_grads=True):
@@ -166,11 +188,14 @@ class RasterizeViews(torch.autograd.Function):
             # the last-contributor record is the other forward's, so the
             # replay runs without it
             ctx.rast.bin_sort(ctx.views, ctx.proj)
-        grads, dvm, _ = ctx.rast.backward(ctx.g, ctx.views, ctx.proj, image, dL_dimage.contiguous(),
-                                          want_gaussian_grads=ctx.want_gauss, use_last=own)
+        # new output arrays (autograd keeps them), the rasterizer's scratch
+        g = ctx.g
+        grads = Grads(g.n, g.sh_degree, 0, 0, g.means.device, ctx.want_gauss,
+                      scratch=ctx.rast.grads_buffers(g, ctx.views, ctx.want_gauss))
+        _, dvm, _ = ctx.rast.backward(g, ctx.views, ctx.proj, image, dL_dimage.contiguous(),
+                                      want_gaussian_grads=ctx.want_gauss, grads=grads, use_last=own)
         if ctx.want_gauss:
-            out = [grads.means.clone(), grads.log_scales.clone(), grads.quats.clone(),
-                   grads.opacity_logits.clone(), grads.sh.clone()]
+            out = [grads.means, grads.log_scales, grads.quats, grads.opacity_logits, grads.sh]
         else:
             out = [None] * 5
         return (*out, dvm, None, None, None)
