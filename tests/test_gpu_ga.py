@@ -352,3 +352,25 @@ def test_weights_upper_median_far_from_the_lower_one(distance):
     torch.cuda.synchronize()
     st = stats.cpu().numpy()
     assert st[1] == np.float32(1.0) and st[2:3].view(np.uint32)[0] == one + distance
+
+
+@pytest.mark.parametrize("count", [1, 127, 128, 129, 384, 511, 512, 513, 1023, 1024, 1025, 1500])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_pairs_of_every_length_around_a_block_of_matches(count, weighted):
+    """Pairs of the same length whose matches start at any offset, one empty pair
+    among them: every distance and the loss against the oracle."""
+    tv, ti, iv, ii, pairs, M = _problem()
+    pairs = pairs[:3]
+    a, b = int(M.offsets[0]), int(M.offsets[1])
+    src = np.resize(M.matches[a:b], (2 * count, 4))
+    offs = np.array([0, count, count, 2 * count], np.int64)
+    w = np.random.default_rng(count).uniform(0.1, 2.0, 2 * count).astype(np.float32) if weighted else None
+    G = synth.Matches(offs, np.ascontiguousarray(src, np.float32), np.ones(2 * count, bool))
+    e_or = OG.distances(ii, iv, pairs, offs, G.matches)
+    kappa = _kappa(ii.astype(np.float64), iv.astype(np.float64), pairs, offs, G.matches.astype(np.float64))
+    e, L, _, _, _, _ = _run_gpu(ii, iv, pairs, G, w)
+    tol = _check_distances(e, e_or, kappa)
+    L_or, _, _ = OG.loss_and_grads(ii, iv, pairs, offs, G.matches, w)
+    # the loss is a weighted mean of the distances
+    ww = np.ones(2 * count) if w is None else w.astype(np.float64)
+    assert abs(L - L_or) <= (ww * tol).sum() / ww.sum() + 1e-5 * L_or
