@@ -27,6 +27,7 @@ constexpr int SS_R = 5;                  // window radius
 constexpr int SS_S1 = SS_T + 2 * SS_R;   // 42: tile + halo where SSIM is formed
 constexpr int SS_IN = SS_T + 4 * SS_R;   // 52: staged input
 constexpr int SS_THREADS = 256;
+constexpr int SS_CH = 3;                 // channels
 constexpr float SS_C1 = 0.0001f, SS_C2 = 0.0009f;
 
 struct SsimLaunch {
@@ -49,14 +50,24 @@ struct SsimSmem {
         float h2[3][SS_S1][SS_T];     // horizontal blurs of a, b, c
     } u;
     float red[2][SS_THREADS / 32];
+    float part[2][SS_CH];             // (split tiles, the first channel's block) each channel's sums
 };
 
-__global__ void __launch_bounds__(SS_THREADS, 4) k_l1_dssim(const SsimLaunch L, const float *__restrict__ image,
-                                                            const float *__restrict__ target, float *__restrict__ grad,
-                                                            float *loss) {
+// Barrier over the channels of a tile (a cluster of blocks).
+__device__ __forceinline__ void tile_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tile_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// BLOCKS: the blocks per SM that the registers leave room for. SPLIT: a cluster of
+// three blocks per tile, one per channel; else a block per tile.
+template <int BLOCKS, bool SPLIT>
+__global__ void __launch_bounds__(SS_THREADS, BLOCKS)
+    k_l1_dssim(const SsimLaunch L, const float *__restrict__ image, const float *__restrict__ target,
+               float *__restrict__ grad, float *loss) {
     extern __shared__ __align__(16) unsigned char ss_raw[];
     SsimSmem &sm = *reinterpret_cast<SsimSmem *>(ss_raw);
-    const long long tile = blockIdx.x;
+    const long long tile = SPLIT ? blockIdx.x / SS_CH : blockIdx.x;
+    const int rank = SPLIT ? blockIdx.x % SS_CH : 0;   // in the cluster
+    if (SPLIT) tile_arrive();
     int v = 0;
     while (v + 1 < L.n_views && L.tile_base[v + 1] <= tile) ++v;
     const int lt = (int)(tile - L.tile_base[v]);
@@ -68,7 +79,7 @@ __global__ void __launch_bounds__(SS_THREADS, 4) k_l1_dssim(const SsimLaunch L, 
     for (int k = 0; k <= 2 * SS_R; ++k) g[k] = L.g[k];
     float acc_s = 0.f, acc_l1 = 0.f;
 
-    for (int ch = 0; ch < 3; ++ch) {
+    for (int ch = rank; ch < (SPLIT ? rank + 1 : SS_CH); ++ch) {
         const float *X = image + L.pix_base[v] + (long long)ch * W * H;
         const float *Y = target + L.pix_base[v] + (long long)ch * W * H;
         float *G = grad + L.pix_base[v] + (long long)ch * W * H;
@@ -221,7 +232,7 @@ __global__ void __launch_bounds__(SS_THREADS, 4) k_l1_dssim(const SsimLaunch L, 
         }
         __syncthreads();
     }
-    // block sums of SSIM and |x - y| over the tile (fixed order), one atomic each
+    // sums of SSIM and |x - y| over the tile (fixed order), one atomic each
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         acc_s += __shfl_xor_sync(0xffffffffu, acc_s, o);
@@ -232,17 +243,31 @@ __global__ void __launch_bounds__(SS_THREADS, 4) k_l1_dssim(const SsimLaunch L, 
         sm.red[1][tid >> 5] = acc_l1;
     }
     __syncthreads();
-    if (tid == 0) {
+    if (SPLIT) {
+        // the channels' sums meet in the first channel's block
+        tile_wait();   // (every block of the cluster has started: its shared memory may be written)
+        if (tid < 2) {
+            float sum = 0.f;
+            for (int w = 0; w < SS_THREADS / 32; ++w) sum += sm.red[tid][w];
+            uint32_t at;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sm.part[tid][rank])), "r"(0));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(at), "f"(sum) : "memory");
+        }
+        __syncwarp();
+        tile_arrive();
+        tile_wait();
+    }
+    if (rank == 0 && tid == 0) {
         float s = 0.f, l = 0.f;
-        for (int w = 0; w < SS_THREADS / 32; ++w) {
-            s += sm.red[0][w];
-            l += sm.red[1][w];
+        for (int w = 0; w < (SPLIT ? SS_CH : SS_THREADS / 32); ++w) {
+            s += SPLIT ? sm.part[0][w] : sm.red[0][w];
+            l += SPLIT ? sm.part[1][w] : sm.red[1][w];
         }
         atomicAdd(&loss[1], l * L.inv_n);
         atomicAdd(&loss[2], s * L.inv_n);
-        // the last block (counted in loss[0], zero before) forms the loss
+        // the last tile (counted in loss[0], zero before) forms the loss
         __threadfence();
-        if (atomicAdd(reinterpret_cast<unsigned int *>(loss), 1u) == gridDim.x - 1) {
+        if (atomicAdd(reinterpret_cast<unsigned int *>(loss), 1u) == L.tile_base[L.n_views] - 1) {
             __threadfence();
             const float l1 = __ldcg(loss + 1), dssim = 1.f - __ldcg(loss + 2);
             loss[2] = dssim;
@@ -278,10 +303,27 @@ int launch_l1_dssim(const int *W, const int *H, int n_views, const float *image,
     L.inv_n = pix > 0 ? (float)(1.0 / (double)pix) : 0.f;
     if (cudaMemsetAsync(loss, 0, 3 * sizeof(float), st) != cudaSuccess) return GS_ERR_CUDA;
     const size_t smem = sizeof(SsimSmem);
-    if (cudaFuncSetAttribute(k_l1_dssim, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    // Few tiles do not fill the chip: up to 1.5 per SM a block per channel (176 tiles
+    // 21 us against 27 with a block per tile, 256 tiles 29 against 27), up to 2 per SM
+    // two blocks per SM with twice the registers (304 tiles 27 us against 31, 400 tiles
+    // 41 against 37).
+    const bool split = 2 * tiles <= 3LL * num_sms(), few = tiles <= 2LL * num_sms();
+    const auto kernel = split ? k_l1_dssim<4, true> : few ? k_l1_dssim<2, false> : k_l1_dssim<4, false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return GS_ERR_CUDA;
     // (views are at least 1x1: there is a tile)
-    k_l1_dssim<<<(unsigned)tiles, SS_THREADS, smem, st>>>(L, image, target, grad, loss);
+    cudaLaunchConfig_t lc = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = SS_CH;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    lc.gridDim = dim3((unsigned)(split ? SS_CH * tiles : tiles));
+    lc.blockDim = dim3(SS_THREADS);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    lc.attrs = at;
+    lc.numAttrs = split ? 1 : 0;
+    if (cudaLaunchKernelEx(&lc, kernel, L, image, target, grad, loss) != cudaSuccess) return GS_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 

@@ -75,3 +75,12 @@ def test_identical_images():
     assert loss[1] == 0 and abs(loss[2]) < 1e-6 and abs(loss[0]) < 1e-6
     # zero up to float32 cancellation in 2x G(b) + y G(c), far below the 1/n scale
     assert np.abs(grads[0]).max() < 1e-3 / ims[0].size
+
+
+@pytest.mark.parametrize("per_2sm, more", [(1, 0), (3, 0), (3, 1), (4, 0), (4, 1)])
+def test_few_tiles_split_by_channel_and_by_registers(per_2sm, more):
+    """Tile counts on both sides of 1.5 and 2 tiles per SM, where the kernel's
+    form changes; tiles cut by the border, views of one tile."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = per_2sm * sms // 2 + more
+    _check(*_images([(31, 32 * (tiles - 2) - 3), (32, 32), (5, 7)], tiles))
