@@ -116,7 +116,8 @@ __device__ __forceinline__ void ga_match(const GaPairGeom &g, float4 q, float w,
 // start and its end leave gaps unless loads cross them: the first matches are asked
 // for before the cameras are, and each thread always has its next four matches on
 // the way (80 registers, six blocks per SM: 60 KB in flight on each). 300 cameras,
-// 21.3M matches, a whole iteration: 94 -> 86 us; eight matches at a time 110 us (four
+// 21.3M matches, a whole iteration: 94 -> 86 us (81 with its four kernels chained, and
+// 22.5 -> 14.3 us for 12 cameras); eight matches at a time 110 us (four
 // blocks), two 96 us, 256 threads 109 us, 64 threads 88 us;
 // one loop body with the matches moved over instead of two bodies 97 us.
 constexpr int GA_UNROLL = 4;
@@ -147,6 +148,8 @@ template <bool WRITE_DIST>
 __global__ void __launch_bounds__(GA_THREADS, GA_PAIR_BLOCKS) k_ga_pairs(const gs_ga_problem P, float *__restrict__ dist,
                                                          float *__restrict__ pair_sums, int32_t *status) {
     __shared__ float s_red[GA_THREADS / 32][11];
+    grid_dependency_wait();
+    launch_dependents();
     const float4 *__restrict__ M4 = reinterpret_cast<const float4 *>(P.matches);
     const float *__restrict__ Wt = P.weights;
     for (long long m = blockIdx.x; m < P.n_pairs; m += gridDim.x) {
@@ -242,6 +245,8 @@ constexpr int GA_TOTAL_THREADS = 1024;
 
 __global__ void __launch_bounds__(GA_TOTAL_THREADS) k_ga_total(long long n_pairs, float *pair_sums, float *loss) {
     __shared__ float s_we[GA_TOTAL_THREADS / 32], s_w[GA_TOTAL_THREADS / 32];
+    grid_dependency_wait();
+    launch_dependents();
     float we = 0.f, w = 0.f;
     for (long long m = threadIdx.x; m < n_pairs; m += GA_TOTAL_THREADS) {
         we += pair_sums[m * GS_GA_PAIR_FLOATS + 9];
@@ -291,6 +296,8 @@ __global__ void __launch_bounds__(GA_CAM_THREADS) k_ga_cams(const gs_ga_problem 
                                                             const int32_t *__restrict__ cam_pairs, float *loss,
                                                             float *d_intr, float *d_vm, const GaStepArgs S) {
     __shared__ float s_red16[GA_CAM_THREADS / 32][16];
+    grid_dependency_wait();
+    launch_dependents();
     // 1 / sum of all weights, left by k_ga_total in the pad slot of row 0
     const float invW = P.n_pairs > 0 ? pair_sums[GS_GA_PAIR_FLOATS - 1] : 0.f;
     const int c = blockIdx.x;
@@ -414,6 +421,8 @@ __device__ __forceinline__ void rot6_fwd(const float *a, Rot6 &r) {
 }
 
 __global__ void k_ga_apply(const GaStepArgs S, int n, float *intr, float *vm, int32_t *step) {
+    grid_dependency_wait();
+    launch_dependents();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c == 0) step[0] += 1;
     if (c >= n) return;
@@ -975,14 +984,14 @@ int launch_ga_epipolar(const gs_ga_problem &P, float *dist, float *pair_sums, co
                        cudaStream_t st) {
     if (P.n_pairs > 0) {
         const unsigned grid = ga_pairs_grid(P.n_pairs);
-        if (dist) k_ga_pairs<true><<<grid, GA_THREADS, 0, st>>>(P, dist, pair_sums, status);
-        else k_ga_pairs<false><<<grid, GA_THREADS, 0, st>>>(P, dist, pair_sums, status);
+        if (dist) launch_chained(k_ga_pairs<true>, grid, GA_THREADS, 0, st, P, dist, pair_sums, status);
+        else launch_chained(k_ga_pairs<false>, grid, GA_THREADS, 0, st, P, dist, pair_sums, status);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
     }
-    k_ga_total<<<1, GA_TOTAL_THREADS, 0, st>>>(P.n_pairs, pair_sums, loss);
+    launch_chained(k_ga_total, 1, GA_TOTAL_THREADS, 0, st, P.n_pairs, pair_sums, loss);
     if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
     if (d_intr && d_vm)
-        k_ga_cams<false><<<P.n_cams, GA_CAM_THREADS, 0, st>>>(P, pair_sums, cam_offsets, cam_pairs, loss, d_intr,
+        launch_chained(k_ga_cams<false>, P.n_cams, GA_CAM_THREADS, 0, st, P, pair_sums, cam_offsets, cam_pairs, loss, d_intr,
                                                                d_vm, GaStepArgs{});
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
@@ -1006,15 +1015,15 @@ int launch_ga_step(const gs_ga_state &s, const gs_ga_problem &P, float *pair_sum
     S.lnb1 = (float)log(s.beta1);
     S.lnb2 = (float)log(s.beta2);
     S.focal = s.optimise_focal;
-    k_ga_apply<<<(s.n_cams + 127) / 128, 128, 0, st>>>(S, s.n_cams, s.intrinsics, s.viewmats, s.step);
+    launch_chained(k_ga_apply, (s.n_cams + 127) / 128, 128, 0, st, S, s.n_cams, s.intrinsics, s.viewmats, s.step);
     if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
     if (P.n_pairs > 0) {
-        k_ga_pairs<false><<<ga_pairs_grid(P.n_pairs), GA_THREADS, 0, st>>>(P, nullptr, pair_sums, status);
+        launch_chained(k_ga_pairs<false>, ga_pairs_grid(P.n_pairs), GA_THREADS, 0, st, P, nullptr, pair_sums, status);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
     }
-    k_ga_total<<<1, GA_TOTAL_THREADS, 0, st>>>(P.n_pairs, pair_sums, loss);
+    launch_chained(k_ga_total, 1, GA_TOTAL_THREADS, 0, st, P.n_pairs, pair_sums, loss);
     if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-    k_ga_cams<true><<<P.n_cams, GA_CAM_THREADS, 0, st>>>(P, pair_sums, cam_offsets, cam_pairs, loss, nullptr,
+    launch_chained(k_ga_cams<true>, P.n_cams, GA_CAM_THREADS, 0, st, P, pair_sums, cam_offsets, cam_pairs, loss, nullptr,
                                                           nullptr, S);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }

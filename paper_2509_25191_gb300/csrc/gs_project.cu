@@ -50,6 +50,8 @@ __global__ void __launch_bounds__(PF_THREADS) k_project_fwd(const Launch L, cons
     constexpr int K = (DEG + 1) * (DEG + 1);
     static_assert(!TMA || DEG == 3, "the staged path is for 48-float SH rows");
     __shared__ __align__(1024) ProjStage S[1];   // (removed by the compiler where unused)
+    grid_dependency_wait();
+    launch_dependents();
     const long long gid0 = (long long)blockIdx.x * PF_THREADS;
     const long long gid = gid0 + threadIdx.x;
     // a block is "full" when its 128 threads are valid Gaussians of one
@@ -276,8 +278,8 @@ int launch_project(const Launch &L, int deg, const gs_gaussians *g, const float 
                      encode_tmap_2d(&ma, g->sh, 48, (uint64_t)g->n, 192, 32, PF_THREADS, CU_TENSOR_MAP_SWIZZLE_128B) &&
                      encode_tmap_2d(&mb, g->sh, 48, (uint64_t)g->n, 192, 16, PF_THREADS, CU_TENSOR_MAP_SWIZZLE_64B) &&
                      encode_tmap_2d(&mp, proj, 16, (uint64_t)L.n_slots, 64, 16, PF_THREADS, CU_TENSOR_MAP_SWIZZLE_64B);
-#define GS_PF(D, T) k_project_fwd<D, T><<<nb, PF_THREADS, 0, st>>>(L, g->means, g->log_scales, g->quats, \
-        g->opacity_logits, g->sh, viewmats, intr, p, ma, mb, mp, status)
+#define GS_PF(D, T) launch_chained(k_project_fwd<D, T>, nb, PF_THREADS, 0, st, L, g->means, g->log_scales, \
+        g->quats, g->opacity_logits, g->sh, viewmats, intr, p, ma, mb, mp, status)
     switch (deg) {
     case 0: GS_PF(0, false); break;
     case 1: GS_PF(1, false); break;

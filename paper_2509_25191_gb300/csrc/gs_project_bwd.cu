@@ -834,22 +834,18 @@ int launch_project_bwd(const Launch &L, int deg, const gs_gaussians *g, const fl
     k_project_bwd<D, G, Z><<<nblk, PB_THREADS, dyn, st>>>(                                                         \
         L, g->means, g->log_scales, g->quats, g->opacity_logits, g->sh, viewmats, intr, p, g2, out->means,        \
         out->log_scales, out->quats, out->opacity_logits, out->sh, out->pose_partials)
+    // (without parameter gradients nothing is written ahead of the kernel's wait)
+#define GS_PB_POSE(D, Z)                                                                                           \
+    launch_chained(k_project_bwd<D, false, Z>, nblk, PB_THREADS, dyn, st, L, g->means, g->log_scales, g->quats,   \
+                   g->opacity_logits, g->sh, viewmats, intr, p, g2, out->means, out->log_scales, out->quats,      \
+                   out->opacity_logits, out->sh, out->pose_partials)
     // one-view calls with parameter gradients and overlap_prev: a programmatic
     // dependent of the kernel ahead (the raster backward in a step), so that
     // each block zeroes its rows while that kernel's tail still runs
 #define GS_PB_EARLY(D)                                                                                             \
     do {                                                                                                           \
-        cudaLaunchConfig_t lc = {};                                                                                \
-        cudaLaunchAttribute at[1];                                                                                 \
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;                                            \
-        at[0].val.programmaticStreamSerializationAllowed = 1;                                                     \
-        lc.gridDim = dim3(nblk);                                                                                   \
-        lc.blockDim = dim3(PB_THREADS);                                                                            \
-        lc.dynamicSmemBytes = dyn;                                                                                 \
-        lc.stream = st;                                                                                            \
-        lc.attrs = at;                                                                                             \
-        lc.numAttrs = 1;                                                                                           \
-        if (cudaLaunchKernelEx(&lc, k_project_bwd<D, true, true>, L, g->means, g->log_scales, g->quats,           \
+        if (launch_chained(k_project_bwd<D, true, true>, nblk, PB_THREADS, dyn, st, L, g->means, g->log_scales,   \
+                           g->quats,                                                                              \
                                g->opacity_logits, g->sh, viewmats, intr, p, g2, out->means, out->log_scales,      \
                                out->quats, out->opacity_logits, out->sh, out->pose_partials) != cudaSuccess)      \
             return GS_ERR_CUDA;                                                                                    \
@@ -897,14 +893,15 @@ int launch_project_bwd(const Launch &L, int deg, const gs_gaussians *g, const fl
         // the pose-only backward reads a Gaussian's parameters only in its
         // contributing views already (per-thread path)
         switch (deg) {
-        case 0: if (compact) GS_PB(0, false, true); else GS_PB(0, false, false); break;
-        case 1: if (compact) GS_PB(1, false, true); else GS_PB(1, false, false); break;
-        case 2: if (compact) GS_PB(2, false, true); else GS_PB(2, false, false); break;
-        case 3: if (compact) GS_PB(3, false, true); else GS_PB(3, false, false); break;
+        case 0: if (compact) GS_PB_POSE(0, true); else GS_PB_POSE(0, false); break;
+        case 1: if (compact) GS_PB_POSE(1, true); else GS_PB_POSE(1, false); break;
+        case 2: if (compact) GS_PB_POSE(2, true); else GS_PB_POSE(2, false); break;
+        case 3: if (compact) GS_PB_POSE(3, true); else GS_PB_POSE(3, false); break;
         default: return GS_ERR_UNSUPPORTED;
         }
     }
 #undef GS_PB
+#undef GS_PB_POSE
 #undef GS_PB_EARLY
 #undef GS_PBV
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
@@ -918,6 +915,8 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float *__restrict__ p
                                                      float *__restrict__ out_twist) {
     __shared__ float s[12][256];
     const int v = blockIdx.x;
+    grid_dependency_wait();
+    launch_dependents();
     float acc[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) acc[c] = 0.f;
@@ -962,7 +961,7 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float *__restrict__ p
 
 int launch_pose_reduce(int n_views, const float *partials, int nblk, const float *viewmats, float *out_rt,
                        float *out_twist, cudaStream_t st) {
-    k_pose_reduce<<<n_views, 256, 0, st>>>(partials, nblk, viewmats, out_rt, out_twist);
+    launch_chained(k_pose_reduce, n_views, 256, 0, st, partials, nblk, viewmats, out_rt, out_twist);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 

@@ -40,11 +40,11 @@ from .autograd import Rasterizer
 
 
 class GraphStep:
-    # project 1, bin/sort 4 (count, scan, scatter, sort), render 1, the zeroing of
+    # project 1, bin/sort 5 (clear, count, scan, scatter, sort), render 1, the zeroing of
     # the backward's accumulators 1 (a kernel with overlap_prev), raster bwd 1,
     # projection bwd 1, pose 1; the L1 loss is part of the raster backward, the
     # L1 + D-SSIM loss adds 1 kernel
-    KERNELS_FIXED = 10
+    KERNELS_FIXED = 11
     SORT_CAP = 4096   # tiles above it may be split (one more kernel where a view has that many Gaussians)
     # the calls of a step, in order (the stages of run()'s events)
     STAGES = {"l1": ("gs_project", "gs_bin_sort", "gs_render_fwd", "gs_rasterize_bwd_l1", "gs_project_bwd",
@@ -57,7 +57,7 @@ class GraphStep:
         return self.STAGES[self.loss_kind]
 
     def kernels_per_step(self) -> int:
-        """Kernels of this library that one step launches: the fixed ten, the
+        """Kernels of this library that one step launches: the fixed eleven, the
         D-SSIM loss kernel, the split of large tiles where a view has Gaussians
         enough for one, and, when the image has fewer than 16 tiles per SM but
         more regions than get a block at once (four per SM), the tile orderings
