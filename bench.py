@@ -43,11 +43,11 @@ UNIT = "Mpix/s"
 # backward. The kernels' own arithmetic (gs_render.cu): every pair that
 # passes the pixel gate evaluates the exponent (dx, dy, 3 mul + 2 fma, o*G,
 # clamp/threshold: 10 ops + 1 ex2); a composited pair adds 9 in the forward
-# (1-alpha, T update, weight, 3 fma) and 34 in the backward (the recomputed
-# accumulation, dL/dalpha, and the pixel's terms of the nine sums).
+# (1-alpha, T update, weight, 3 fma) and 50 in the backward (colour/alpha/
+# conic/mean gradients and the recomputed accumulation).
 FWD_FLOPS_EVAL, BWD_FLOPS_EVAL = 12, 40
 FWD_OPS_EVAL, FWD_OPS_COMP = 10, 9
-BWD_OPS_EVAL, BWD_OPS_COMP = 10, 34
+BWD_OPS_EVAL, BWD_OPS_COMP = 10, 50
 FP32_LANES_PER_SM = 128
 # tile shapes the autotuner tries on the large secondary workloads (uneven
 # scenes, dense step), where each candidate step is expensive to build: the

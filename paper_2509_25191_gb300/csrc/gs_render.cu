@@ -22,18 +22,18 @@
 // everything behind Gaussian i from the forward image,
 //   S_i = sum_{j>i} c_j alpha_j T_j + T_final bg = image - sum_{j<=i} c_j alpha_j T_j,
 // so that dL/dalpha_i = T_i (c_i . g) - (S_i . g) / (1 - alpha_i).
-// Per-Gaussian gradients (mean2D, 2D covariance, opacity, colour) are linear in
-// two numbers per pixel, the weight w = alpha T and dp = dL/dalpha o G: a visit
-// only stores these two for its pixels in a per-warp buffer; when eight visits
-// are pending, four lanes per visit add up the moments of dp over the patch and
-// the sums of w times the upstream gradient. The moments are summed over the
-// block in shared memory and turned into the nine gradients once per (region,
-// Gaussian), which go to the per-slot grad2d record with one vector atomic per
-// float4.
+// Per-Gaussian gradients (mean2D, 2D covariance, opacity, colour) are summed over a
+// warp through a shared-memory transpose: a warp writes the 9 values of up to
+// three consecutive visits as rows of a per-warp buffer (one column per lane),
+// then 27 lanes each add one row with 16-byte loads; then over the block in
+// shared memory, and into the per-slot grad2d record with one vector atomic
+// per float4.
 // Both kernels run a thread's two pixels through packed float2 arithmetic
 // (f32x2 fma/mul/add, one instruction for both), branch-free: a pixel that
 // does not composite a Gaussian contributes zeros.
 #include "gs_common.cuh"
+
+#include <type_traits>
 
 namespace gsk {
 
@@ -84,25 +84,28 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 
 // The raster kernels' unit of work: RW x RH pixels of a TW x TH tile, BS =
-// RW RH / 2 threads. Tiles of more than 256 pixels are walked in 16x16 parts by
-// 128-thread blocks that each go through the tile's list and stage only what
-// reaches their part. The barriers around a batch make a block's warps wait
-// for the one with the most visits: with a 512-thread block on a 32x32 tile of
-// the 1M-Gaussian view the slowest warp had 1.51 times the mean warp's visits
-// per batch (1.34 per tile), with 16x16 parts 1.24 (1.15). Testing a Gaussian
-// once per part costs a few instructions against the ~100 of a visit, and the
-// coarser tiles keep binning and the sort cheap. Smaller parts would balance
-// better still, but each adds its own sum to a Gaussian's gradient, in float32.
-// With the sums over pending visits below: backward 309 -> 267 us on the 1M
-// view; steps 687 -> 668 us (1M view), 4169 -> 4062 (16-view orbit), 6329 -> 6070
-// (16 uneven views).
-template <int TW, int TH>
+// RW RH / 2 threads.
+// Tiles of more than 256 pixels are walked in 16x16 parts by 128-thread blocks
+// that each go through the tile's list and stage only what reaches their part. The
+// barriers around a batch make a block's warps wait for the one with the most
+// visits: with a 512-thread block on a 32x32 tile of the 1M-Gaussian view the
+// slowest warp had 1.51 times the mean warp's visits per batch (1.34 per tile),
+// with 16x16 parts 1.24 (1.15). Testing a Gaussian once per part costs a few
+// instructions against the ~100 of a visit, and the coarser tiles keep binning and
+// the sort cheap. The image does not depend on it.
+template <int TW_, int TH_, bool PARTED>
 struct Region {
-    static constexpr bool SPLIT = TW * TH > 256;
+    static constexpr int TW = TW_, TH = TH_;
+    static constexpr bool SPLIT = PARTED && TW * TH > 256;
     static constexpr int RW = SPLIT ? 16 : TW, RH = SPLIT ? 16 : TH;
     static constexpr int SX = TW / RW, PARTS = SX * (TH / RH);
     static constexpr int BS = RW * RH / 2, WARPS = BS / 32;
+    using Mask = std::conditional_t<(WARPS > 8), unsigned short, unsigned char>;   // a bit per warp
 };
+template <int TW, int TH>
+using FwdRegion = Region<TW, TH, true>;
+template <int TW, int TH>
+using BwdRegion = Region<TW, TH, true>;
 
 struct TileInfo {
     int view;
@@ -118,14 +121,13 @@ struct TileInfo {
 // Positions are relative to the enclosing 32x32-pixel block (every supported
 // tile nests in one), so a pixel's arithmetic is the same for every tile
 // shape and the image is bit-identical across shapes.
-template <int TW, int TH>
+template <typename R>
 __device__ __forceinline__ TileInfo tile_info(const Launch &L, int tile, int part) {
-    using R = Region<TW, TH>;
     TileInfo ti;
     ti.view = view_of_tile(L, tile);
     const ViewDesc &vd = L.v[ti.view];
     const int lt = tile - vd.tile_base;
-    const int rx = (lt % vd.Gx) * TW + (part % R::SX) * R::RW, ry = (lt / vd.Gx) * TH + (part / R::SX) * R::RH;
+    const int rx = (lt % vd.Gx) * R::TW + (part % R::SX) * R::RW, ry = (lt / vd.Gx) * R::TH + (part / R::SX) * R::RH;
     const int w = (int)threadIdx.x >> 5, l = (int)threadIdx.x & 31;
     ti.px = rx + (w % (R::RW / 8)) * 8 + (l & 7);
     ti.py0 = ry + (w / (R::RW / 8)) * 8 + (l >> 3);
@@ -198,16 +200,17 @@ __device__ __forceinline__ void count_pairs(int *counters, int at, unsigned int 
 // One staged Gaussian: its three float4 lie together (48 bytes apart, an odd
 // number of 16-byte bank groups: no conflicts on the stores), so that a visit
 // reads them at one address.
-template <int TW, int TH>
+template <typename R>
 __device__ __forceinline__ void stage_one(const Launch &L, const float4 *__restrict__ proj,
                                           const unsigned int *__restrict__ ids, int index, int k, const TileInfo &ti,
-                                          float4 *s_st, unsigned char *s_mask) {
+                                          float4 *s_st, typename R::Mask *s_mask, float2 *s_ad) {
     float4 xy, con, rgb;
     stage(proj, ids[index], index, ti.ox, ti.oy, xy, con, rgb);
     s_st[3 * k] = xy;
     s_st[3 * k + 1] = con;
     s_st[3 * k + 2] = rgb;
-    s_mask[k] = (unsigned char)warp_mask<Region<TW, TH>::RW, Region<TW, TH>::RH>(xy, con, L.alpha_min, ti.tbx, ti.tby);
+    if (s_ad) s_ad[k] = make_float2(con.x * (-2.f * LN2), con.z * (-2.f * LN2));
+    s_mask[k] = (typename R::Mask)warp_mask<R::RW, R::RH>(xy, con, L.alpha_min, ti.tbx, ti.tby);
 }
 
 // Stage the next batch of a tile's instances [pos, end) that reach the block's
@@ -223,16 +226,16 @@ struct Pack {
     unsigned int ballot[32];   // [test j][warp]
     int next;
 };
-template <int TW, int TH>
+template <typename R>
 __device__ __forceinline__ int stage_batch(const Launch &L, const float4 *__restrict__ proj,
                                            const unsigned int *__restrict__ ids, int &pos, int end, int per,
-                                           const TileInfo &ti, float4 *s_st, unsigned char *s_mask, Pack *pk) {
-    using R = Region<TW, TH>;
+                                           const TileInfo &ti, float4 *s_st, typename R::Mask *s_mask, Pack *pk,
+                                           float2 *s_ad = nullptr) {
     constexpr int BS = R::BS;
     if constexpr (R::PARTS == 1) {
         for (int h = 0; h < per; ++h) {
             const int k = threadIdx.x + h * BS;
-            if (k < end - pos) stage_one<TW, TH>(L, proj, ids, pos + k, k, ti, s_st, s_mask);
+            if (k < end - pos) stage_one<R>(L, proj, ids, pos + k, k, ti, s_st, s_mask, s_ad);
         }
         const int nb = min(per * BS, end - pos);
         pos += nb;
@@ -274,7 +277,7 @@ __device__ __forceinline__ int stage_batch(const Launch &L, const float4 *__rest
             const int k = base + __popc(bal & ((1u << lane) - 1u));
             const int i = pos + j * BS + threadIdx.x;
             if (bal >> lane & 1u) {
-                if (k < cap) stage_one<TW, TH>(L, proj, ids, i, k, ti, s_st, s_mask);
+                if (k < cap) stage_one<R>(L, proj, ids, i, k, ti, s_st, s_mask, s_ad);
                 else if (k == cap) pk->next = i;   // the first that did not fit starts the next batch
             }
         }
@@ -297,97 +300,32 @@ __device__ __forceinline__ int next_item(int *queue, int items, int *s_item) {
 }
 
 // Shared-memory bytes of one staged Gaussian: position, conic and colour
-// (3 x 16 B) and the warp mask (a byte: at most four warps); the backward adds
-// its nine sums.
-constexpr int FWD_STAGE_BYTES = 49;
-constexpr int BWD_STAGE_BYTES = 85;
-// The backward's per-warp buffer: RED_VISITS pending visits of 32 lanes, a
-// float4 (w, dp of the lane's two pixels) each, and the lanes' upstream
-// gradients (a float4 and a float2 each).
-constexpr int RED_VISITS = 8;
-constexpr int RED_WARP_BYTES = RED_VISITS * 32 * 16 + 32 * 24;
-// Threads per SM the backward's registers are capped for: 896 (72 registers, 30 KB
-// of shared memory per 128 threads): 1M view 670 us a step, against 683 with 1,024
-// (64 registers, and six pending visits to fit) and 671 with 768. The one-warp
-// blocks of 8x8 tiles keep more addresses in registers: 640 (96 registers), 24
-// views of three scenes 6.65 ms against 6.97 with 768 and 7.05 with 896.
-constexpr int bwd_blocks(int threads) { return (threads == 32 ? 640 : 896) / threads; }
-
-// Lane l = 8 q + i owns column i and rows q, q + 4 of its patch. Its entry in a
-// row of 32 is at red_at(l), + 4 exchanged in odd visits: the lanes of a
-// quarter-warp that read column i of two visits and four q's then hit the
-// eight 16-byte bank groups once each.
-__device__ __forceinline__ int red_at(int l) { return (l & 24) | ((l & 7) ^ (l >> 3)); }
-
-// Sums over the pending visits' patches, by four lanes per visit: lane 4 s + q
-// of the warp adds up rows q and q + 4 of visit s (lane .x = row q, .y = row
-// q + 4) from its buffer row. u is formed per pixel as in the walk (moments
-// about a fixed point would cancel: u is small on a thin Gaussian's ridge where
-// dx and beta dy are not); dy is constant over a row. The nine sums
-//   sum dp (1, u, dy, u^2, u dy, dy^2), sum w (g_r, g_g, g_b)
-// are folded over the four lanes, each keeping two (lane 0 three), and added to
-// the Gaussian's sums over the block in s_g. k: the staged index of visit s.
-__device__ __forceinline__ void reduce_visits(const float4 *__restrict__ buf, const float4 *__restrict__ g4,
-                                              const float2 *__restrict__ g2, int npend, int k, float px0, float py0,
-                                              const float4 *s_st, float *s_g) {
-    const int lane = threadIdx.x & 31, s = lane >> 2, q = lane & 3;
-    const float4 *row = buf + s * 32 + 8 * q;
-    const int odd = (s & 1) << 2;
-    const float4 xy = s_st[3 * k];
-    const float beta = s_st[3 * k + 1].y;
-    const float y0 = py0 + (float)q;
-    const float2 dy = make_float2(y0 - xy.y, (y0 + 4.f) - xy.y);
-    float2 S0 = make_float2(0.f, 0.f), su = S0, suu = S0, CR = S0, CG = S0, CB = S0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float4 v = row[i ^ (q | odd)];
-        const float4 gv = g4[8 * q + (i ^ q)];
-        const float2 gb = g2[8 * q + (i ^ q)];
-        const float2 w = make_float2(v.x, v.y), dp = make_float2(v.z, v.w);
-        const float dx = (px0 + (float)i) - xy.x;
-        const float2 u = __ffma2_rn(f2(beta), dy, f2(dx));
-        const float2 t = __fmul2_rn(dp, u);
-        S0 = __fadd2_rn(S0, dp);
-        su = __fadd2_rn(su, t);
-        suu = __ffma2_rn(t, u, suu);
-        CR = __ffma2_rn(w, make_float2(gv.x, gv.y), CR);
-        CG = __ffma2_rn(w, make_float2(gv.z, gv.w), CG);
-        CB = __ffma2_rn(w, gb, CB);
-    }
-    const float2 sy = __fmul2_rn(dy, S0), suy = __fmul2_rn(dy, su), syy = __fmul2_rn(dy, sy);
-    const float t[9] = {S0.x + S0.y, su.x + su.y, sy.x + sy.y, suu.x + suu.y, suy.x + suy.y, syy.x + syy.y,
-                        CR.x + CR.y, CG.x + CG.y, CB.x + CB.y};
-    // sums j and j + 4 change hands between the lanes of a pair, then j and
-    // j + 2: lane q ends with sums 4 (q & 1) + (q & 2) + {0, 1}
-    const bool b0 = q & 1, b1 = q & 2;
-    float r[4], z[2], t8 = t[8];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) r[j] = (b0 ? t[j + 4] : t[j]) + __shfl_xor_sync(0xffffffffu, b0 ? t[j] : t[j + 4], 1);
-    t8 += __shfl_xor_sync(0xffffffffu, t8, 1);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) z[j] = (b1 ? r[j + 2] : r[j]) + __shfl_xor_sync(0xffffffffu, b1 ? r[j] : r[j + 2], 2);
-    t8 += __shfl_xor_sync(0xffffffffu, t8, 2);
-    if (s < npend) {
-        float *dst = s_g + 9 * k;
-        float *two = dst + 4 * (q & 1) + (q & 2);
-        atomicAdd(two, z[0]);
-        atomicAdd(two + 1, z[1]);
-        if (q == 0) atomicAdd(dst + 8, t8);
-    }
-}
+// (3 x 16 B) and the warp mask; the backward adds the conic's natural-log
+// terms (8 B) and the per-Gaussian gradient sums (9 floats).
+template <typename R>
+constexpr int FWD_STAGE_BYTES = 48 + (int)sizeof(typename R::Mask);
+template <typename R>
+constexpr int BWD_STAGE_BYTES = 92 + (int)sizeof(typename R::Mask);
+// The backward's per-warp reduction buffer: RED_SLOTS visits x 9 values as
+// rows of 32 lane columns, row pitch RED_PITCH floats (16-byte aligned rows;
+// the 4-float pad puts the 8 lanes of a quarter-warp reading 16 bytes of 8
+// different rows on 8 disjoint groups of 4 banks).
+constexpr int RED_SLOTS = 3;
+constexpr int RED_PITCH = 36;
+constexpr int RED_WARP_FLOATS = RED_SLOTS * 9 * RED_PITCH;
 
 template <int TW, int TH>
-__global__ void __launch_bounds__(Region<TW, TH>::BS, 1024 / Region<TW, TH>::BS)
+__global__ void __launch_bounds__(FwdRegion<TW, TH>::BS, 1024 / FwdRegion<TW, TH>::BS)
     k_render_fwd(const Launch L, const float4 *__restrict__ proj, const int2 *__restrict__ ranges,
                  const unsigned int *__restrict__ ids, const int *__restrict__ order, int *__restrict__ counters,
                  float *__restrict__ image, int *__restrict__ last_contrib, int *__restrict__ tile_work) {
     // the staged batch (L.fwd_batch Gaussians per thread) in dynamic shared memory
-    using R = Region<TW, TH>;
+    using R = FwdRegion<TW, TH>;
     constexpr int BS = R::BS;
     const int NB = L.fwd_batch * BS;
     extern __shared__ float4 s_dyn[];
     float4 *s_st = s_dyn;
-    unsigned char *s_mask = reinterpret_cast<unsigned char *>(s_st + 3 * NB);
+    typename R::Mask *s_mask = reinterpret_cast<typename R::Mask *>(s_st + 3 * NB);
     __shared__ int s_item;
     __shared__ Pack s_pack;
     // the backward's accumulators that follow (zeroed by a programmatic
@@ -401,7 +339,7 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, 1024 / Region<TW, TH>::BS)
         const int tile = order[item / R::PARTS];
         // (a tile of one part: no other block adds to its record)
         if (R::PARTS == 1 && tile_work && threadIdx.x == 0) tile_work[tile] = 0;
-        const TileInfo ti = tile_info<TW, TH>(L, tile, item % R::PARTS);
+        const TileInfo ti = tile_info<R>(L, tile, item % R::PARTS);
         const int2 r = abort ? make_int2(0, 0) : ranges[tile];
         // lane .x = pixel (px, py0), lane .y = pixel (px, py0 + 4)
         float2 T = f2(1.f), CR = f2(0.f), CG = f2(0.f), CB = f2(0.f);
@@ -414,7 +352,7 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, 1024 / Region<TW, TH>::BS)
         const float2 PCY = make_float2(ti.pcy0, ti.pcy0 + 4.f);
         for (int pos = r.x; pos < r.y;) {
             if (__syncthreads_count(am0 == INF && am1 == INF) == BS) break;
-            const int nb = stage_batch<TW, TH>(L, proj, ids, pos, r.y, L.fwd_batch, ti, s_st, s_mask, &s_pack);
+            const int nb = stage_batch<R>(L, proj, ids, pos, r.y, L.fwd_batch, ti, s_st, s_mask, &s_pack);
             // the warp walks only the staged Gaussians that may reach its patch:
             // 32 masks per ballot, then the set bits in order
             for (int k0 = 0; k0 < nb; k0 += 32) {
@@ -488,26 +426,26 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, 1024 / Region<TW, TH>::BS)
 // is composited, and the warp and the block stop at their pixels' largest
 // end instead of walking on to saturation or the end of the list.
 template <int TW, int TH, bool COUNT, bool LAST>
-__global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>::BS))
+__global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH>::BS)
     k_render_bwd(const Launch L, const float4 *__restrict__ proj, const int2 *__restrict__ ranges,
                  const unsigned int *__restrict__ ids, const int *__restrict__ order, int *__restrict__ counters,
                  const float *__restrict__ image, const float *__restrict__ dL_dimage,
                  const int *__restrict__ last_contrib, float4 *__restrict__ grad2d,
                  const float *__restrict__ l1_target, float *__restrict__ l1_loss, float l1_inv_n,
                  float *__restrict__ l1_part) {
-    // dynamic shared memory: the per-warp buffers of pending visits and the
-    // lanes' upstream gradients, then the staged batch (L.bwd_batch Gaussians
-    // per thread): positions, conics and colours, the sums over the block
-    // (pitch 9, odd: no bank conflicts) and the warp masks
-    using R = Region<TW, TH>;
+    // dynamic shared memory: the per-warp reduction buffers, then the staged
+    // batch (L.bwd_batch Gaussians per thread): positions, conics and colours,
+    // the conic's A and D (natural-log units), the per-Gaussian gradient sums
+    // (pitch 9, odd: no bank conflicts) and warp masks
+    using R = BwdRegion<TW, TH>;
     constexpr int BS = R::BS;
     const int NB = L.bwd_batch * BS;
     extern __shared__ float4 s_dyn[];
-    float4 *s_g4 = s_dyn + (BS / 32) * RED_VISITS * 32;
-    float2 *s_g2 = reinterpret_cast<float2 *>(s_g4 + BS);
-    float4 *s_st = reinterpret_cast<float4 *>(s_g2 + BS);
-    float *s_g = reinterpret_cast<float *>(s_st + 3 * NB);
-    unsigned char *s_mask = reinterpret_cast<unsigned char *>(s_g + 9 * NB);
+    float *s_red = reinterpret_cast<float *>(s_dyn);
+    float4 *s_st = s_dyn + R::WARPS * RED_WARP_FLOATS / 4;
+    float2 *s_ad = reinterpret_cast<float2 *>(s_st + 3 * NB);
+    float *s_g = reinterpret_cast<float *>(s_ad + NB);
+    typename R::Mask *s_mask = reinterpret_cast<typename R::Mask *>(s_g + 9 * NB);
     __shared__ int s_item;
     __shared__ Pack s_pack;
     __shared__ float s_l1[R::WARPS];
@@ -516,19 +454,22 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>:
     // it zeroes its gradient rows there, then waits for this grid to finish
     launch_dependents();
     if (counters[CNT_ABORT]) return;
-    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
+    const int lane = threadIdx.x & 31;
     const unsigned int wbit = 1u << (threadIdx.x >> 5);
-    // this warp's pending visits, and this lane's entry in the next one's row
-    float4 *rb = s_dyn + (threadIdx.x >> 5) * RED_VISITS * 32;
-    const int red0 = red_at(lane);
-    int red_next = red0;
+    // this warp's buffer: row 9 s + j holds value j of the warp's pending
+    // visit s (s < RED_SLOTS), column l that of lane l
+    float *rb = s_red + (threadIdx.x >> 5) * RED_WARP_FLOATS;
+    // at a flush, lane 9 s + j (j < 9) adds row 9 s + j: value j of pending
+    // visit s, whose staged index lane s holds
+    const int red_j = lane % 9, red_s = lane / 9;
+    const float4 *red_row = reinterpret_cast<const float4 *>(rb + lane * RED_PITCH);
     for (int k = threadIdx.x; k < 9 * NB; k += BS) s_g[k] = 0.f;
     float l1_sum = 0.f;   // with l1_target: this thread's sum of |image - target|
     const int items = L.n_tiles * R::PARTS;
     __syncthreads();   // the sums are zero
     for (int item = blockIdx.x; item < items; item = next_item(counters + CNT_Q_BWD, items, &s_item)) {
         const int tile = order[item / R::PARTS];
-        const TileInfo ti = tile_info<TW, TH>(L, tile, item % R::PARTS);
+        const TileInfo ti = tile_info<R>(L, tile, item % R::PARTS);
         const int2 r = ranges[tile];
         const ViewDesc &vd = L.v[ti.view];
         const long long hw = (long long)vd.W * vd.H;
@@ -573,31 +514,39 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>:
         const float2 PCY = make_float2(ti.pcy0, ti.pcy0 + 4.f);
         float2 T = f2(1.f), CG = f2(0.f);
         unsigned int n_eval = 0, n_comp = 0;
-        // the upstream gradients for the sums over visits (read by this warp only)
-        s_g4[warp0 + red0] = make_float4(GR.x, GR.y, GG.x, GG.y);
-        s_g2[warp0 + red0] = GB;
         // the warp's pending visits (warp-uniform) and, in lane s, the staged
         // index of pending visit s
         int npend = 0, kpend = 0;
+        // add the pending visits' rows to their Gaussians' sums in s_g (each
+        // row over the 32 lanes: two f32x2 chains over 8 16-byte loads, then
+        // the two lanes of the pair)
+        auto flush = [&]() {
+            __syncwarp();
+            const int kk = __shfl_sync(0xffffffffu, kpend, red_s);
+            if (lane < 9 * npend) {
+                float4 v = red_row[0];
+                float2 sa = make_float2(v.x, v.y), sb = make_float2(v.z, v.w);
+#pragma unroll
+                for (int i = 1; i < 8; ++i) {
+                    v = red_row[i];
+                    sa = __fadd2_rn(sa, make_float2(v.x, v.y));
+                    sb = __fadd2_rn(sb, make_float2(v.z, v.w));
+                }
+                sa = __fadd2_rn(sa, sb);
+                atomicAdd(&s_g[9 * kk + red_j], sa.x + sa.y);
+            }
+            npend = 0;
+            __syncwarp();   // the buffer is free for the next visits
+        };
         for (int pos = r.x; pos < r.y;) {
             if (__syncthreads_count(LAST ? pos >= endm : done0 && done1) == BS) break;
-            const int nb = stage_batch<TW, TH>(L, proj, ids, pos, r.y, L.bwd_batch, ti, s_st, s_mask, &s_pack);
-            // the warp takes only the staged Gaussians that may reach its patch, in
-            // order: 32 masks per ballot, then the set bits; the pending visits are
-            // summed when the buffer is full and once at the end of the batch
-            int k0 = -32;
-            unsigned int hits = 0u;
-            for (;;) {
-                bool last = false;
-                while (!hits) {
-                    k0 += 32;
-                    // the end of the batch, or the warp's pixels have all stopped
-                    last = k0 >= nb || __all_sync(0xffffffffu, LAST ? __float_as_int(s_st[3 * k0 + 2].w) >= endm
-                                                                    : done0 && done1);
-                    if (last) break;
-                    hits = __ballot_sync(0xffffffffu, k0 + lane < nb && (s_mask[k0 + lane] & wbit));
-                }
-                if (!last) {
+            const int nb = stage_batch<R>(L, proj, ids, pos, r.y, L.bwd_batch, ti, s_st, s_mask, &s_pack, s_ad);
+            for (int k0 = 0; k0 < nb; k0 += 32) {
+                // the warp's pixels have all stopped
+                if (__all_sync(0xffffffffu, LAST ? __float_as_int(s_st[3 * k0 + 2].w) >= endm : done0 && done1)) break;
+                // only the staged Gaussians that may reach this warp's patch, in order
+                unsigned int hits = __ballot_sync(0xffffffffu, k0 + lane < nb && (s_mask[k0 + lane] & wbit));
+                while (hits) {
                     const int k = k0 + __ffs(hits) - 1;
                     hits &= hits - 1;
                     const float4 xy = s_st[3 * k], con = s_st[3 * k + 1], c = s_st[3 * k + 2];
@@ -647,6 +596,8 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>:
                     const float2 w = __fmul2_rn(ac, T);
                     const float2 Told = T;
                     T = Tn;
+                    const float2 ad = s_ad[k];
+                    const float2 g6 = __fmul2_rn(w, GR), g7 = __fmul2_rn(w, GG), g8 = __fmul2_rn(w, GB);
                     // c.g, and C.g accumulated through this Gaussian; S.g = image.g - C.g,
                     // dL/dalpha = T (c.g) - (S.g) / (1 - alpha) (1 - alpha >= 0.01, so
                     // the approximate reciprocal's few-ulp error is far inside the
@@ -656,58 +607,57 @@ __global__ void __launch_bounds__(Region<TW, TH>::BS, bwd_blocks(Region<TW, TH>:
                     const float2 q = __fmul2_rn(__fadd2_rn(CG, NIG), make_float2(rcp_approx(oma.x), rcp_approx(oma.y)));
                     const float2 dla = __ffma2_rn(Told, cgk, q);
                     // alpha = o G unless clamped; G = exp(power), power = -1/2 d^T Q d,
-                    // Q the conic, d = pixel - mean: d alpha / d power = alpha where it
-                    // is composited unclamped, else 0. With v = Q d, d power / d mean = v
-                    // and d power / d Sigma' = v v^T / 2, i.e. (v0^2/2, v0 v1, v1^2/2) for
-                    // (a, b, c); summing these well-scaled terms (reduce_visits) avoids
-                    // the ill-conditioned conic -> covariance conversion of summed
-                    // conic gradients.
-                    const float2 dp = __fmul2_rn(dla, make_float2(oG.x <= L.alpha_max ? ac.x : 0.f,
-                                                                  oG.y <= L.alpha_max ? ac.y : 0.f));
-                    if (!LAST && !__any_sync(0xffffffffu, cp0 || cp1)) continue;
-                    rb[red_next] = make_float4(w.x, w.y, dp.x, dp.y);
-                    red_next = (red_next + 32) ^ 4;
-                    kpend = lane == npend ? k : kpend;
-                    if (++npend < RED_VISITS) continue;
-                } else if (npend == 0) {
-                    break;
+                    // Q the conic, d = pixel - mean. With v = Q d = (A u, A beta u + D dy)
+                    // from the staged form, d power / d mean = v and d power / d Sigma' =
+                    // v v^T / 2, i.e. (v0^2/2, v0 v1, v1^2/2) for (a, b, c); summing these
+                    // well-scaled terms avoids the ill-conditioned conic -> covariance
+                    // conversion of summed conic gradients. The halves of the (a) and (c)
+                    // sums are applied once, at the flush. Gu = G where the pixel composites
+                    // an unclamped alpha, else 0; d alpha / d power = o Gu.
+                    const bool un0 = cp0 && oG.x <= L.alpha_max, un1 = cp1 && oG.y <= L.alpha_max;
+                    const float2 g5 = __fmul2_rn(dla, make_float2(un0 ? G.x : 0.f, un1 ? G.y : 0.f));
+                    const float2 dp = __fmul2_rn(f2(con.w), g5);
+                    const float2 v0 = __fmul2_rn(f2(ad.x), u);
+                    const float2 v1 = __ffma2_rn(v0, f2(con.y), __fmul2_rn(f2(ad.y), dy));
+                    const float2 g0 = __fmul2_rn(dp, v0), g1 = __fmul2_rn(dp, v1);
+                    const float2 g2 = __fmul2_rn(g0, v0), g3 = __fmul2_rn(g0, v1), g4 = __fmul2_rn(g1, v1);
+                    if (__any_sync(0xffffffffu, cp0 || cp1)) {
+                        // gradient of this thread's pixels w.r.t. (x, y, a, b, c, o, r, g, b),
+                        // as column `lane` of the next pending visit's rows
+                        float *wr = rb + npend * (9 * RED_PITCH) + lane;
+                        wr[0 * RED_PITCH] = g0.x + g0.y;
+                        wr[1 * RED_PITCH] = g1.x + g1.y;
+                        wr[2 * RED_PITCH] = g2.x + g2.y;
+                        wr[3 * RED_PITCH] = g3.x + g3.y;
+                        wr[4 * RED_PITCH] = g4.x + g4.y;
+                        wr[5 * RED_PITCH] = g5.x + g5.y;
+                        wr[6 * RED_PITCH] = g6.x + g6.y;
+                        wr[7 * RED_PITCH] = g7.x + g7.y;
+                        wr[8 * RED_PITCH] = g8.x + g8.y;
+                        kpend = lane == npend ? k : kpend;
+                        if (++npend == RED_SLOTS) flush();
+                    }
                 }
-                __syncwarp();
-                reduce_visits(rb, s_g4 + warp0, s_g2 + warp0, npend, __shfl_sync(0xffffffffu, kpend, lane >> 2),
-                              ti.pcx - (float)(lane & 7), ti.pcy0 - (float)(lane >> 3), s_st, s_g);
-                npend = 0;
-                red_next = red0;
-                __syncwarp();   // the buffer is free for the next visits
-                if (last) break;
             }
+            if (npend) flush();   // (warp-uniform) before the batch's sums leave
             __syncthreads();
-            // the batch's Gaussians that got a sum: the nine gradients, with
-            // A, D the conic's terms in natural-log units and v = (A u, beta A u + D dy)
+            // flush this batch's per-Gaussian sums
             for (int h = 0; h < L.bwd_batch; ++h) {
                 const int k = threadIdx.x + h * BS;
                 if (k < nb) {
                     float *sg = s_g + 9 * k;
-                    float t[9];
-                    unsigned int any = 0u;
-#pragma unroll
-                    for (int j = 0; j < 9; ++j) {
-                        t[j] = sg[j];
-                        any |= __float_as_uint(t[j]);
-                    }
-                    if (any & 0x7fffffffu) {
-                        const float4 con = s_st[3 * k + 1];
-                        const float A = con.x * (-2.f * LN2), D = con.z * (-2.f * LN2), beta = con.y;
-                        const float g0 = A * t[1], g1 = fmaf(beta, g0, D * t[2]);
-                        const float g2 = A * A * t[3], ad = A * t[4];                   // sum dp v0^2, sum dp v0 dy
-                        const float g3 = fmaf(beta, g2, D * ad);                        // sum dp v0 v1
-                        const float g4 = fmaf(beta, g3, D * fmaf(beta, ad, D * t[5]));  // sum dp v1^2
+                    const float a0 = sg[0], a1 = sg[1], a2 = 0.5f * sg[2], a3 = sg[3];
+                    const float a4 = 0.5f * sg[4];
+                    const float a5 = sg[5], a6 = sg[6], a7 = sg[7], a8 = sg[8];
+                    if (a0 != 0.f || a1 != 0.f || a2 != 0.f || a3 != 0.f || a4 != 0.f || a5 != 0.f || a6 != 0.f ||
+                        a7 != 0.f || a8 != 0.f) {
                         float4 *dst = grad2d + 3ull * ids[__float_as_int(s_st[3 * k + 2].w)];
-                        atomicAdd(dst, make_float4(g0, g1, 0.5f * g2, g3));
-                        atomicAdd(dst + 1, make_float4(0.5f * g4, t[0] / con.w, t[6], t[7]));
-                        atomicAdd(dst + 2, make_float4(t[8], 0.f, 0.f, 0.f));
-#pragma unroll
-                        for (int j = 0; j < 9; ++j) sg[j] = 0.f;
+                        atomicAdd(dst, make_float4(a0, a1, a2, a3));
+                        atomicAdd(dst + 1, make_float4(a4, a5, a6, a7));
+                        atomicAdd(dst + 2, make_float4(a8, 0.f, 0.f, 0.f));
                     }
+#pragma unroll
+                    for (int j = 0; j < 9; ++j) sg[j] = 0.f;
                 }
             }
         }
@@ -805,7 +755,10 @@ static bool order_by_work(const Launch &L, const gs_bins *b) {
 // kernel keeps at least four blocks per SM), so neither an order nor a queue
 // matters, and the launches that prepare them are left out (4 to 5 us each in a
 // step of 120 us).
-static bool all_at_once(long long items) { return items <= 4LL * num_sms(); }
+template <int TW, int TH>
+static bool all_at_once(const Launch &L) {
+    return (long long)L.n_tiles * FwdRegion<TW, TH>::PARTS <= 4LL * num_sms();
+}
 // where the forward records the replay lengths: the caller's kept record,
 // else tile_scratch (this call only)
 static int *work_record(const gs_bins *b) { return b->tile_work ? b->tile_work : b->tile_scratch; }
@@ -874,9 +827,9 @@ __global__ void __launch_bounds__(1024) k_order_by_work(int *__restrict__ work, 
 
 template <int TW, int TH>
 static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, float *image, cudaStream_t st) {
-    using R = Region<TW, TH>;
+    using R = FwdRegion<TW, TH>;
     static int blocks_per_sm[5];
-    const size_t smem = (size_t)FWD_STAGE_BYTES * L.fwd_batch * R::BS;
+    const size_t smem = (size_t)FWD_STAGE_BYTES<R> * L.fwd_batch * R::BS;
     const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_fwd<TW, TH>, R::BS, smem,
                                                                           L.fwd_batch, blocks_per_sm),
                               max(1LL, (long long)L.n_tiles * R::PARTS));
@@ -888,7 +841,7 @@ static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, fl
     // several parts collects the largest of their lengths, from zero.
     const long long items = (long long)L.n_tiles * R::PARTS;
     const bool ordered = order_by_work(L, b);
-    if (ordered && b->tile_work && !all_at_once(items)) {
+    if (ordered && b->tile_work && !all_at_once<TW, TH>(L)) {
         k_order_by_work<<<1, 1024, 0, st>>>(b->tile_work, reinterpret_cast<const int2 *>(b->tile_ranges),
                                             (int)L.n_tiles, b->tile_order, true, b->counters + CNT_Q_FWD);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
@@ -908,18 +861,24 @@ static int launch_fwd_t(const Launch &L, const float *proj, const gs_bins *b, fl
 
 template <int TW, int TH, bool COUNT, bool LAST>
 static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, const float *image,
-                        const float *dL_dimage, const L1Loss &l1, float *grad2d, bool queue_reset, cudaStream_t st) {
-    using R = Region<TW, TH>;
+                        const float *dL_dimage, const L1Loss &l1, float *grad2d, cudaStream_t st) {
+    using R = BwdRegion<TW, TH>;
     static int blocks_per_sm[5];
-    const size_t smem = (size_t)BWD_STAGE_BYTES * L.bwd_batch * R::BS + (size_t)RED_WARP_BYTES * R::WARPS;
+    const size_t smem = (size_t)BWD_STAGE_BYTES<R> * L.bwd_batch * R::BS + sizeof(float) * RED_WARP_FLOATS * R::WARPS;
+    const long long items = (long long)L.n_tiles * R::PARTS;
     const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_bwd<TW, TH, COUNT, LAST>, R::BS,
                                                                           smem, L.bwd_batch, blocks_per_sm),
-                              max(1LL, (long long)L.n_tiles * R::PARTS));
+                              max(1LL, items));
     // the queue head, and the count of blocks that have added to the loss
     static_assert(CNT_L1_DONE == CNT_Q_BWD + 1, "reset together");
-    if (!queue_reset && grid < (long long)L.n_tiles * R::PARTS &&
-        cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, 2 * sizeof(int), st) != cudaSuccess)
+    if (order_by_work(L, b) && !all_at_once<TW, TH>(L)) {
+        // by the replay lengths that the forward recorded
+        k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false,
+                                            b->counters + CNT_Q_BWD);
+        if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
+    } else if (grid < items && cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, 2 * sizeof(int), st) != cudaSuccess) {
         return GS_ERR_CUDA;
+    }
     // the blocks' parts of the loss lie behind the work record (tile_scratch is
     // 5 ints per tile; the grid has at most PARTS <= 4 blocks per tile)
     static_assert(R::PARTS <= 4, "one part of the loss per block fits tile_scratch");
@@ -938,19 +897,11 @@ static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, co
 template <int TW, int TH>
 static int launch_bwd_t(const Launch &L, const float *proj, const gs_bins *b, const float *image,
                         const float *dL_dimage, const L1Loss &l1, float *grad2d, cudaStream_t st) {
-    if (b->last_contrib) {
-        // the forward recorded each tile's replay length
-        const bool ordered = order_by_work(L, b) && !all_at_once((long long)L.n_tiles * Region<TW, TH>::PARTS);
-        if (ordered) {
-            k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false,
-                                                b->counters + CNT_Q_BWD);
-            if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-        }
-        return L.count_pairs ? launch_bwd_c<TW, TH, true, true>(L, proj, b, image, dL_dimage, l1, grad2d, ordered, st)
-                             : launch_bwd_c<TW, TH, false, true>(L, proj, b, image, dL_dimage, l1, grad2d, ordered, st);
-    }
-    return L.count_pairs ? launch_bwd_c<TW, TH, true, false>(L, proj, b, image, dL_dimage, l1, grad2d, false, st)
-                         : launch_bwd_c<TW, TH, false, false>(L, proj, b, image, dL_dimage, l1, grad2d, false, st);
+    if (b->last_contrib)
+        return L.count_pairs ? launch_bwd_c<TW, TH, true, true>(L, proj, b, image, dL_dimage, l1, grad2d, st)
+                             : launch_bwd_c<TW, TH, false, true>(L, proj, b, image, dL_dimage, l1, grad2d, st);
+    return L.count_pairs ? launch_bwd_c<TW, TH, true, false>(L, proj, b, image, dL_dimage, l1, grad2d, st)
+                         : launch_bwd_c<TW, TH, false, false>(L, proj, b, image, dL_dimage, l1, grad2d, st);
 }
 
 int launch_render_fwd(const Launch &L, const float *proj, const gs_bins *b, float *image, cudaStream_t st) {
