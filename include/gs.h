@@ -88,8 +88,10 @@ typedef struct gs_config {
                              results are the same bit for bit. */
     int fwd_batch;        /* [2] Gaussians each thread stages per shared-memory batch in gs_render_fwd:
                              1, 2 or 4 (a batch is fwd_batch x threads Gaussians; a block has a thread
-                             per two pixels of its tile, or of a 16x16 part of a tile above 256) */
-    int bwd_batch;        /* [1] the same for gs_rasterize_bwd: 1 or 2. Neither changes the image; the
+                             per two pixels of its tile, or of a 16x16 part of a tile above 256
+                             pixels) */
+    int bwd_batch;        /* [1] the same for gs_rasterize_bwd, whose blocks have a thread per two
+                             pixels of the whole tile: 1 or 2. Neither changes the image; the
                              2D gradients change only in the order of their float additions. */
     int overlap_prev;     /* [0] nonzero: gs_rasterize_bwd(_l1) and the one-view gs_project_bwd with
                              parameter gradients are launched as programmatic dependents of the kernel

@@ -9,8 +9,9 @@
 //   and the pixel stops.
 //
 // Both kernels are persistent: blocks pull regions of tiles from an atomic
-// queue over tile_order (largest tiles first). A region is the tile, or for
-// 32x32 and 32x16 tiles one of its 16x16 quarters or halves (see Region).
+// queue over tile_order (largest tiles first). A region is the tile, or in the
+// forward for 32x32 and 32x16 tiles one of its 16x16 quarters or halves (see
+// Region).
 // Each thread owns two pixels and each warp an 8x8-pixel patch of the region; a
 // tile's instances are staged through shared memory in batches (the number per
 // thread chosen at launch: by default two in the forward, one in the backward),
@@ -85,14 +86,19 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // The raster kernels' unit of work: RW x RH pixels of a TW x TH tile, BS =
 // RW RH / 2 threads.
-// Tiles of more than 256 pixels are walked in 16x16 parts by 128-thread blocks
-// that each go through the tile's list and stage only what reaches their part. The
-// barriers around a batch make a block's warps wait for the one with the most
-// visits: with a 512-thread block on a 32x32 tile of the 1M-Gaussian view the
+// Forward: tiles of more than 256 pixels are walked in 16x16 parts by 128-thread
+// blocks that each go through the tile's list and stage only what reaches their
+// part. The barriers around a batch make a block's warps wait for the one with the
+// most visits: with a 512-thread block on a 32x32 tile of the 1M-Gaussian view the
 // slowest warp had 1.51 times the mean warp's visits per batch (1.34 per tile),
 // with 16x16 parts 1.24 (1.15). Testing a Gaussian once per part costs a few
 // instructions against the ~100 of a visit, and the coarser tiles keep binning and
 // the sort cheap. The image does not depend on it.
+// Backward: a block per tile. Parts would each add a sum of their own to a
+// Gaussian's gradient, in float32, and a long thin Gaussian's gradients along its
+// long axis are small differences of those sums: with parts single elements of the
+// quaternion gradients of a 16-view orbit (32x16 tiles) moved by 6.7e-4 of the rms,
+// with one sum per tile by 2.3e-4 (2.1e-4 between two runs).
 template <int TW_, int TH_, bool PARTED>
 struct Region {
     static constexpr int TW = TW_, TH = TH_;
@@ -105,7 +111,7 @@ struct Region {
 template <int TW, int TH>
 using FwdRegion = Region<TW, TH, true>;
 template <int TW, int TH>
-using BwdRegion = Region<TW, TH, true>;
+using BwdRegion = Region<TW, TH, false>;
 
 struct TileInfo {
     int view;
@@ -751,10 +757,11 @@ static int raster_blocks_per_sm(K kernel, int threads, size_t smem, int batch, i
 static bool order_by_work(const Launch &L, const gs_bins *b) {
     return b->last_contrib && L.n_tiles > 0 && L.n_tiles < 16LL * num_sms();
 }
-// Few regions: every one gets a resident block of its own at once (each raster
-// kernel keeps at least four blocks per SM), so neither an order nor a queue
-// matters, and the launches that prepare them are left out (4 to 5 us each in a
-// step of 120 us).
+// Few tiles: every region of the forward and every tile of the backward gets a
+// resident block of its own at once (the forward keeps eight of its blocks per SM,
+// the backward at least one 32x32 tile, two 32x16 tiles or four smaller ones),
+// so neither an order nor a queue matters, and the launches that prepare them are
+// left out (4 to 5 us each in a step of 120 us).
 template <int TW, int TH>
 static bool all_at_once(const Launch &L) {
     return (long long)L.n_tiles * FwdRegion<TW, TH>::PARTS <= 4LL * num_sms();

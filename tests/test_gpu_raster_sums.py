@@ -51,3 +51,44 @@ def test_one_pixel_gives_a_rank_one_covariance_gradient(tile, use_last):
         off = np.abs(4 * a[on] * c[on] / b[on] ** 2 - 1)
         assert off.max() <= 10 * EPS, ((px, py), off.max() / EPS)
     assert seen > 50 and thin > 5
+
+
+@pytest.mark.parametrize("use_last", [True, False])
+@pytest.mark.parametrize("tile", [(16, 16), (32, 16), (32, 32)])
+def test_a_tile_adds_one_sum(tile, use_last):
+    """A round Gaussian on the centre of the middle tile column, one large
+    upstream gradient of each sign at mirrored pixels of its tiles: equal
+    weights, so these tiles' colour sums cancel to exactly 0 before they leave
+    the tile. What is left are the single pixels of the other tiles, whose sum in
+    any order is within (n - 1) half-ulps of their absolute sum; added in
+    parts, the large terms would cost them seventeen bits."""
+    tw, th = tile
+    W, H = 3 * tw, 96
+    sc = synth.uniform_box_scene(0, 1, sh_degree=0)
+    sc.means[:] = (0.0, 0.0, 2.0)
+    sc.log_scales[:] = np.log(1.0)
+    sc.quats[:] = (1.0, 0.0, 0.0, 0.0)
+    sc.opacity_logits[:] = 0.0
+    vw = synth._views(np.concatenate([np.eye(3).reshape(-1), np.zeros(3)]), 60.0, W, H, 0, 1)
+    g, views = _lib.Gaussians.from_scene(sc), _lib.Views.from_synth(vw)
+    rast = Rasterizer(tile=tile)
+    image, proj = rast.forward(g, views)
+    rng = np.random.default_rng(5)
+    pairs = np.zeros((3, H, W), np.float32)
+    single = []
+    for ty in range(H // th):
+        # mirrored columns of the middle tile column, both of one row
+        y, d = ty * th + int(rng.integers(th)), int(rng.integers(tw // 4, tw // 2))
+        pairs[:, y, W // 2 + d] = 131072.0
+        pairs[:, y, W // 2 - 1 - d] = -131072.0
+        for tx in (0, 2):
+            up = np.zeros((3, H, W), np.float32)
+            up[:, ty * th + int(rng.integers(th)), tx * tw + int(rng.integers(tw))] = rng.uniform(0.5, 1.0, 3)
+            single.append(up)
+    dev = lambda u: torch.as_tensor(u.reshape(-1), device="cuda")
+    terms = np.stack([_backward(rast, views, proj, image, dev(u), use_last)[0, 6:9] for u in single])
+    assert (np.abs(terms) > 0).all()
+    want, room = terms.sum(0), (len(terms) - 1) * EPS * np.abs(terms).sum(0)
+    for _ in range(8):
+        got = _backward(rast, views, proj, image, dev(pairs + np.sum(single, 0)), use_last)[0, 6:9]
+        assert (np.abs(got - want) <= room).all(), (got, want, room)
