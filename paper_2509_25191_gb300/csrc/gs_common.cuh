@@ -49,7 +49,7 @@ struct Launch {
 
 // The mean L1 loss folded into the raster backward: with target set, the
 // upstream gradient of each image value is sign(image - target) * inv_n and
-// the loss inv_n * sum |image - target| is added to *loss.
+// *loss, which is zero before, becomes inv_n * sum |image - target|.
 struct L1Loss {
     const float *target = nullptr;
     float *loss = nullptr;
@@ -63,7 +63,6 @@ enum {
     CNT_Q_FWD = 2,       // work queue heads
     CNT_Q_BWD = 3,
     CNT_Q_SORT = 4,
-    CNT_L1_DONE = 4,     // (after the sort) blocks of the raster backward whose part of the loss is written
     CNT_RUN_RES = 5,     // runs of split large tiles listed for the sort
     CNT_MAX_TILE = 6,    // largest per-tile count
     CNT_Q_SPLIT = 7      // queue head of the large-tile split

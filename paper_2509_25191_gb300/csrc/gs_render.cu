@@ -670,34 +670,38 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
         if (COUNT) count_pairs(counters, 12, n_eval, n_comp);
     }
     if (l1_loss) {
-        // the block's part of the loss
+        // a sum over the block, in thread 0
+        auto block_sum = [&](float x) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) l1_sum += __shfl_xor_sync(0xffffffffu, l1_sum, o);
-        if (lane == 0) s_l1[threadIdx.x >> 5] = l1_sum;
-        __syncthreads();
-        if (threadIdx.x < 32) {
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (lane == 0) s_l1[threadIdx.x >> 5] = x;
+            __syncthreads();
             float t = 0.f;
-            for (int w = 0; w < R::WARPS; ++w) t += s_l1[w];
-            if (!l1_part) {
-                if (lane == 0) atomicAdd(l1_loss, t * l1_inv_n);
-                return;
-            }
-            // the last block to get here adds up the parts (a thousand or more
-            // of them: an atomic sum would round each addition to the whole)
-            int done = 0;
-            if (lane == 0) {
-                __stcg(l1_part + blockIdx.x, t);
-                __threadfence();
-                done = atomicAdd(counters + CNT_L1_DONE, 1);
-            }
-            if (__shfl_sync(0xffffffffu, done, 0) != (int)gridDim.x - 1) return;
-            __threadfence();
-            float sum = 0.f;
-            for (int i = lane; i < (int)gridDim.x; i += 32) sum += __ldcg(l1_part + i);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane == 0) *l1_loss = sum * l1_inv_n;
+            if (threadIdx.x == 0)
+                for (int w = 0; w < R::WARPS; ++w) t += s_l1[w];
+            return t;
+        };
+        const float t = block_sum(l1_sum);
+        if (!l1_part) {
+            if (threadIdx.x == 0) atomicAdd(l1_loss, t * l1_inv_n);
+            return;
         }
+        // the last block to get here adds up the blocks' parts (hundreds of them:
+        // an atomic sum would round each addition to the whole). The blocks are
+        // counted in the loss's own word, which is zero before this kernel
+        if (threadIdx.x == 0) {
+            __stcg(l1_part + blockIdx.x, t);
+            __threadfence();
+            s_item = atomicAdd(reinterpret_cast<unsigned int *>(l1_loss), 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!s_item) return;
+        __threadfence();
+        float sum = 0.f;
+#pragma unroll 8
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += BS) sum += __ldcg(l1_part + i);
+        sum = block_sum(sum);
+        if (threadIdx.x == 0) *l1_loss = sum * l1_inv_n;
     }
 }
 
@@ -785,7 +789,7 @@ __device__ __forceinline__ int work_bucket(int w) {
 }
 // With reset, the record is zeroed after it has been read (the forward that
 // follows takes the maximum over a tile's pixels into it). The kernel's queue
-// head and the word after it are cleared too.
+// head is cleared too.
 __global__ void __launch_bounds__(1024) k_order_by_work(int *__restrict__ work, const int2 *__restrict__ ranges,
                                                         int n_tiles, int *__restrict__ order, bool reset, int *queue) {
     __shared__ int s_cnt[1024];
@@ -798,7 +802,7 @@ __global__ void __launch_bounds__(1024) k_order_by_work(int *__restrict__ work, 
         return r.y - r.x;
     };
     s_cnt[tid] = 0;
-    if (tid < 2) queue[tid] = 0;
+    if (tid == 0) *queue = 0;
     __syncthreads();
     for (int t = tid; t < n_tiles; t += 1024) atomicAdd(&s_cnt[work_bucket(predicted(t))], 1);
     __syncthreads();
@@ -876,22 +880,22 @@ static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, co
     const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_bwd<TW, TH, COUNT, LAST>, R::BS,
                                                                           smem, L.bwd_batch, blocks_per_sm),
                               max(1LL, items));
-    // the queue head, and the count of blocks that have added to the loss
-    static_assert(CNT_L1_DONE == CNT_Q_BWD + 1, "reset together");
     if (order_by_work(L, b) && !all_at_once<TW, TH>(L)) {
         // by the replay lengths that the forward recorded
         k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false,
                                             b->counters + CNT_Q_BWD);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-    } else if (grid < items && cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, 2 * sizeof(int), st) != cudaSuccess) {
+    } else if (grid < items && cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, sizeof(int), st) != cudaSuccess) {
         return GS_ERR_CUDA;
     }
     // the blocks' parts of the loss lie behind the work record (tile_scratch is
-    // 5 ints per tile; the grid has at most PARTS <= 4 blocks per tile)
+    // 5 ints per tile, the grid at most one block per region). Two blocks per SM or
+    // more: their ordered sum has an error of 1e-7 where the atomic additions, each
+    // rounded to the whole, reach 1e-6, and costs a step 1 to 2 us (304 tiles of 16x16
+    // 84.4 -> 86.2 us, 2,170 of them 450 -> 452; 2,500 tiles of 8x8 173 -> 178). Fewer
+    // blocks add to the loss with atomics.
     static_assert(R::PARTS <= 4, "one part of the loss per block fits tile_scratch");
-    // (the ordered sum costs a small launch about 2 us: only where the blocks
-    // are many, or more of them than one per tile)
-    const bool many = grid > (R::PARTS > 1 ? 4 : 8) * num_sms();
+    const bool many = grid >= 2 * num_sms();
     float *l1_part = l1.loss && b->tile_scratch && many
                          ? reinterpret_cast<float *>(b->tile_scratch + L.n_tiles) : nullptr;
     k_render_bwd<TW, TH, COUNT, LAST><<<grid, R::BS, smem, st>>>(
