@@ -37,7 +37,8 @@ class Rasterizer:
         self.bins = None
         self.status = None
         self.fixed_capacity = False   # set for graph capture: never read back
-        self._grads = None
+        self._scratch = None          # 2D gradients and pose partials of a backward
+        self._grads = None            # the same with parameter gradients (Rasterizer.backward)
         self._count = None            # pinned host word and event of the count's readback
         self.last_instances = None
         self.generation = 0           # counts bin_sort calls: which forward the tile lists belong to
@@ -120,11 +121,18 @@ class Rasterizer:
             self.render(views, proj, self.bins, image)
         return image, proj
 
+    def scratch_buffers(self, g: Gaussians, views: Views):
+        """The scratch of a backward: a Grads without parameter gradients."""
+        key = (g.n, views.num_slots(), views.n, g.means.device)
+        if self._scratch is None or self._scratch[0] != key:
+            self._scratch = (key, Grads(g.n, 0, views.num_slots(), views.n, g.means.device, False))
+        return self._scratch[1]
+
     def grads_buffers(self, g: Gaussians, views: Views, want_gaussian_grads=True):
         key = (g.n, g.sh_degree, views.num_slots(), views.n, want_gaussian_grads, g.means.device)
         if self._grads is None or self._grads[0] != key:
             self._grads = (key, Grads(g.n, g.sh_degree, views.num_slots(), views.n, g.means.device,
-                                      want_gaussian_grads))
+                                      want_gaussian_grads, scratch=self.scratch_buffers(g, views)))
         return self._grads[1]
 
     def backward(self, g: Gaussians, views: Views, proj, image, dL_dimage, want_gaussian_grads=True,
@@ -191,7 +199,7 @@ class RasterizeViews(torch.autograd.Function):
         # new output arrays (autograd keeps them), the rasterizer's scratch
         g = ctx.g
         grads = Grads(g.n, g.sh_degree, 0, 0, g.means.device, ctx.want_gauss,
-                      scratch=ctx.rast.grads_buffers(g, ctx.views, ctx.want_gauss))
+                      scratch=ctx.rast.scratch_buffers(g, ctx.views))
         _, dvm, _ = ctx.rast.backward(g, ctx.views, ctx.proj, image, dL_dimage.contiguous(),
                                       want_gaussian_grads=ctx.want_gauss, grads=grads, use_last=own)
         if ctx.want_gauss:
