@@ -19,9 +19,9 @@
 // Bound by instruction issue, with a barrier after each of the five passes: it
 // needs several blocks per SM to cover them, so a, b, c take the staged inputs'
 // place (the centre pixels are read again from the caches) and registers are
-// capped for four blocks. Two 1237x822 images: 141 us (139 with a blur of x^2 + y^2
-// for (x - y)^2, and then 142 with three blocks, 158 with two); 174 us with five
-// blurs, its own room for a, b, c and two blocks per SM. Error of the gradient
+// capped for four blocks. Two 1237x822 images, back to back: 133 us (137 with a blur of
+// x^2 + y^2 for (x - y)^2, and then 141 with three blocks, 157 with two); 173 us with
+// five blurs, its own room for a, b, c and two blocks per SM. Error of the gradient
 // against 64 bits, five blurs -> (x - y)^2: 2.4e-6 -> 1.9e-6 for images 0.1 apart,
 // 1.2e-5 -> 6.0e-6 for 0.01, 2.5e-4 -> 8.1e-5 for a bright flat image 1e-3 apart.
 #include "gs_common.cuh"
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(SS_THREADS, BLOCKS)
                     da = 2.f * my * (l2 - l1) * rq + 2.f * mx * S * (rd2 - rd1);
                     db = -S * rd2;
                     dc = 2.f * l1 * rq;
-                    if (r >= SS_R && r < SS_R + SS_T && c >= SS_R && c < SS_R + SS_T) acc_s += 1.f - S;
+                    if (r >= SS_R && r < SS_R + SS_T && c >= SS_R && c < SS_R + SS_T) acc_s += S;
                 }
                 sm.in.abc[0][r][c] = da;
                 sm.in.abc[1][r][c] = db;
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(SS_THREADS, BLOCKS)
         }
         __syncthreads();
     }
-    // sums of 1 - SSIM and |x - y| over the tile (fixed order), one atomic each
+    // sums of SSIM and |x - y| over the tile (fixed order), one atomic each
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         acc_s += __shfl_xor_sync(0xffffffffu, acc_s, o);
@@ -269,13 +269,24 @@ __global__ void __launch_bounds__(SS_THREADS, BLOCKS)
             s += SPLIT ? sm.part[0][w] : sm.red[0][w];
             l += SPLIT ? sm.part[1][w] : sm.red[1][w];
         }
+        // The additions to the loss round to the whole, and there are thousands of
+        // them: a full tile with SSIM above 1/2 adds its distance from 1 and is
+        // counted (an image against itself adds nothing but rounding; two 1237x822
+        // images 0.1 apart: error 3e-7 either way, 8e-7 with every distance from 1).
+        constexpr float FULL = SS_CH * SS_T * SS_T;
+        const unsigned int tiles = (unsigned int)L.tile_base[L.n_views];
+        const bool count_ones = tiles < 0x10000u;   // (two 16-bit counts in loss[0], zero before)
+        const bool one = count_ones && W - ox >= SS_T && H - oy >= SS_T && s > 0.5f * FULL;
         atomicAdd(&loss[1], l * L.inv_n);
-        atomicAdd(&loss[2], s * L.inv_n);
-        // the last tile (counted in loss[0], zero before) forms the loss
+        atomicAdd(&loss[2], (one ? s - FULL : s) * L.inv_n);
+        // the last tile forms the loss
         __threadfence();
-        if (atomicAdd(reinterpret_cast<unsigned int *>(loss), 1u) == L.tile_base[L.n_views] - 1) {
+        const unsigned int n = atomicAdd(reinterpret_cast<unsigned int *>(loss), one ? 0x10001u : 1u);
+        if ((count_ones ? n & 0xffffu : n) == tiles - 1) {
             __threadfence();
-            const float l1 = __ldcg(loss + 1), dssim = __ldcg(loss + 2);
+            const float ones = count_ones ? (float)((n >> 16) + (one ? 1u : 0u)) : 0.f;
+            const float l1 = __ldcg(loss + 1), dssim = (1.f - ones * FULL * L.inv_n) - __ldcg(loss + 2);
+            loss[2] = dssim;
             loss[0] = (1.f - L.lambda) * l1 + L.lambda * dssim;
         }
     }
