@@ -164,7 +164,8 @@ __device__ __forceinline__ int count_bucket(int c) { return c <= 0 ? 0 : 32 - __
 // instance total and capacity check, and the work order (tiles by decreasing
 // count bucket). Four neighbouring tiles per thread, 4,096 tiles a round; the
 // lanes of a warp that fall into one bucket take their places with one atomic.
-// Bound by latency (one block): 25 us for 17,360 tiles, 27 with an atomic per tile.
+// Bound by latency (one block): 25 us for 17,360 tiles, 27 with an atomic per tile
+// (both with neighbouring tiles side by side in the work order, below).
 __global__ void __launch_bounds__(1024) k_bin_scan(const Launch L, long long capacity, int *__restrict__ tile_count,
                                                    int2 *__restrict__ ranges, int *__restrict__ order,
                                                    int *__restrict__ counters, int *__restrict__ status) {
@@ -259,19 +260,27 @@ __global__ void __launch_bounds__(1024) k_bin_scan(const Launch L, long long cap
         }
     }
     __syncthreads();
-    for (int base = 0; base < T; base += 4096) {
+    // Thread i places tiles i per .. (i + 1) per, so that neighbours of one bucket lie
+    // a thousand places apart in the work order. Side by side they were rasterized at
+    // the same time, and the backward's sums of a Gaussian that covers them met in
+    // another order on every run: two runs of a 16-view orbit (17,360 tiles) then
+    // differed by 3.0e-7 of the mean gradients' norm, by 1.9e-7 this way (median of 36
+    // pairs), for 0.2 % of the step (3,961 -> 3,968 us; the reads of the ranges are strided).
+    const int per = (T + 1023) / 1024;
+    for (int base = 0; base < per; base += 4) {
         int c[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int t = base + k * 1024 + tid;
-            const int2 r = t < T ? ranges[t] : make_int2(0, 0);
+            const int t = tid * per + base + k;
+            const int2 r = base + k < per && t < T ? ranges[t] : make_int2(0, 0);
             c[k] = r.y - r.x;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int t = base + k * 1024 + tid;
-            const int pos = place(s_base, count_bucket(c[k]), t < T);
-            if (t < T) order[pos] = t;
+            const int t = tid * per + base + k;
+            const bool valid = base + k < per && t < T;
+            const int pos = place(s_base, count_bucket(c[k]), valid);
+            if (valid) order[pos] = t;
         }
     }
 }
