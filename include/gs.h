@@ -138,7 +138,7 @@ typedef struct gs_bins {
     uint64_t *keys_tmp;   /* [capacity] scratch for tiles too large for on-chip sorting */
     int32_t *tile_order;  /* [T] work order: tiles by decreasing instance count */
     int32_t *tile_scratch;/* [5T] scratch (per-tile counters, then the runs of large tiles that
-                             are sorted in pieces, and the blocks' parts of the folded L1 loss) */
+                             are sorted in pieces) */
     int32_t *counters;    /* [GS_NUM_COUNTERS] scratch; counters[0] = instances after the call;
                              int64 at counters+8: pixel-Gaussian pairs evaluated by gs_render_fwd,
                              +10: composited by it, +12/+14: the same for gs_rasterize_bwd */
@@ -307,7 +307,7 @@ int gs_project_bwd(const gs_gaussians *g, const gs_views *views, const gs_config
  * formed in the kernel from image and target (DEVICE, same layout as image)
  * instead of read from a dL_dimage buffer, which is neither needed nor
  * written. loss DEVICE [1] is overwritten with mean |image - target| (block
- * partials added with atomics, so its last bits depend on their order).
+ * partials added with atomics, so its last bit depends on their order).
  * grad2d as in gs_rasterize_bwd. Same errors as gs_rasterize_bwd; GS_ERR_ARG
  * also for a NULL target or loss. */
 int gs_rasterize_bwd_l1(const gs_views *views, const gs_config *cfg, const float *proj, const gs_bins *bins,

@@ -28,7 +28,7 @@ int launch_bin_sort(const Launch &L, const float *proj, const gs_bins *b, int32_
 int launch_render_fwd(const Launch &L, const float *proj, const gs_bins *b, float *image, cudaStream_t st);
 int launch_render_bwd(const Launch &L, const float *proj, const gs_bins *b, const float *image,
                       const float *dL_dimage, const L1Loss &l1, float *grad2d, cudaStream_t st);
-int launch_zero_accumulators(float *grad2d, long long n_floats, float *loss, cudaStream_t st);
+int launch_zero_accumulators(float *grad2d, long long n_floats, const L1Loss &l1, bool early, cudaStream_t st);
 int launch_project_bwd(const Launch &L, int deg, const gs_gaussians *g, const float *viewmats, const float *intr,
                        const float *proj, const float *grad2d, const gs_grads *out, int want_gauss, int nblk,
                        int32_t *status, cudaStream_t st);
@@ -370,7 +370,7 @@ int gs_rasterize_bwd(const gs_views *vw, const gs_config *cfg, const float *proj
     (void)status;   // the raster backward reports nothing on the device
     cudaStream_t st = (cudaStream_t)stream;
     if (L.overlap_prev) {
-        if ((rc = launch_zero_accumulators(grad2d, (long long)GS_GRAD2D_FLOATS * L.n_slots, nullptr, st))) return rc;
+        if ((rc = launch_zero_accumulators(grad2d, (long long)GS_GRAD2D_FLOATS * L.n_slots, L1Loss{}, true, st))) return rc;
     } else if (cudaMemsetAsync(grad2d, 0, sizeof(float) * GS_GRAD2D_FLOATS * (size_t)L.n_slots, st) != cudaSuccess) {
         return GS_ERR_CUDA;
     }
@@ -392,16 +392,13 @@ int gs_rasterize_bwd_l1(const gs_views *vw, const gs_config *cfg, const float *p
     const int64_t count = gs_num_image_floats(vw);
     if (count < 1) return GS_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    if (L.overlap_prev) {
-        if ((rc = launch_zero_accumulators(grad2d, (long long)GS_GRAD2D_FLOATS * L.n_slots, loss, st))) return rc;
-    } else if (cudaMemsetAsync(grad2d, 0, sizeof(float) * GS_GRAD2D_FLOATS * (size_t)L.n_slots, st) != cudaSuccess ||
-               cudaMemsetAsync(loss, 0, sizeof(float), st) != cudaSuccess) {
-        return GS_ERR_CUDA;
-    }
     L1Loss l1;
     l1.target = target;
     l1.loss = loss;
+    l1.carry = reinterpret_cast<float *>(b->counters + CNT_L1_CARRY);
     l1.inv_n = 1.f / (float)count;
+    if ((rc = launch_zero_accumulators(grad2d, (long long)GS_GRAD2D_FLOATS * L.n_slots, l1, L.overlap_prev, st)))
+        return rc;
     return launch_render_bwd(L, proj, b, image, nullptr, l1, grad2d, st);
 }
 

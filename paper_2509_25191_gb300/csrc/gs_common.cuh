@@ -52,7 +52,7 @@ struct Launch {
 // *loss, which is zero before, becomes inv_n * sum |image - target|.
 struct L1Loss {
     const float *target = nullptr;
-    float *loss = nullptr;
+    float *loss = nullptr, *carry = nullptr;   // (carry: what the additions to the loss round away)
     float inv_n = 0.f;
 };
 
@@ -61,11 +61,12 @@ enum {
     CNT_INSTANCES = 0,   // total tile instances
     CNT_ABORT = 1,       // nonzero: capacity exceeded, skip the rest
     CNT_Q_FWD = 2,       // work queue heads
-    CNT_Q_BWD = 3,
+    CNT_Q_BWD = 3,       // (left at zero by the binning and by every raster backward)
     CNT_Q_SORT = 4,
     CNT_RUN_RES = 5,     // runs of split large tiles listed for the sort
     CNT_MAX_TILE = 6,    // largest per-tile count
-    CNT_Q_SPLIT = 7      // queue head of the large-tile split
+    CNT_Q_SPLIT = 7,     // queue head of the large-tile split
+    CNT_L1_CARRY = 7     // (a float; zeroed by every call that uses it) carry of the folded L1 loss
 };
 
 // ---------------------------------------------------------------------------

@@ -431,6 +431,27 @@ __global__ void __launch_bounds__(FwdRegion<TW, TH>::BS, 1024 / FwdRegion<TW, TH
 // last composited one), so every Gaussian that passes the alpha test there
 // is composited, and the warp and the block stop at their pixels' largest
 // end instead of walking on to saturation or the end of the list.
+// Add a block's part to the loss. Every addition rounds to the whole: hundreds of
+// them leave an error of 1e-6. With a carry word (zero before the kernel) what an
+// addition rounds away, which the old value and the part give exactly, goes there,
+// and what has gathered there is added again: an error of 1e-7, and no block has to be
+// the last to know it (a count of the blocks, an ordered sum by the last one and
+// the fences for it made the kernel slower as a whole, 1M view 301 -> 315 us at 16x16
+// tiles, 319 -> 334 at 32x32). What an infinite sum rounds away is not a number
+// and is dropped.
+__device__ __forceinline__ void add_loss(float *loss, float part, float *carry) {
+    auto add = [&](float x) {
+        const float old = atomicAdd(loss, x), sum = old + x;
+        const float lost = fabsf(old) >= fabsf(x) ? x - (sum - old) : old - (sum - x);
+        return fabsf(lost) < __int_as_float(0x7f800000) ? lost : 0.f;
+    };
+    const float lost = add(part);
+    if (!carry) return;
+    atomicAdd(carry, lost);
+    const float more = atomicExch(carry, 0.f);
+    if (more != 0.f) atomicAdd(carry, add(more));
+}
+
 template <int TW, int TH, bool COUNT, bool LAST>
 __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH>::BS)
     k_render_bwd(const Launch L, const float4 *__restrict__ proj, const int2 *__restrict__ ranges,
@@ -438,7 +459,7 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
                  const float *__restrict__ image, const float *__restrict__ dL_dimage,
                  const int *__restrict__ last_contrib, float4 *__restrict__ grad2d,
                  const float *__restrict__ l1_target, float *__restrict__ l1_loss, float l1_inv_n,
-                 float *__restrict__ l1_part) {
+                 float *__restrict__ l1_carry) {
     // dynamic shared memory: the per-warp reduction buffers, then the staged
     // batch (L.bwd_batch Gaussians per thread): positions, conics and colours,
     // the conic's A and D (natural-log units), the per-Gaussian gradient sums
@@ -670,55 +691,33 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
         if (COUNT) count_pairs(counters, 12, n_eval, n_comp);
     }
     if (l1_loss) {
-        // a sum over the block, in thread 0
-        auto block_sum = [&](float x) {
+        // the block's part of the loss
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0) s_l1[threadIdx.x >> 5] = x;
-            __syncthreads();
-            float t = 0.f;
-            if (threadIdx.x == 0)
-                for (int w = 0; w < R::WARPS; ++w) t += s_l1[w];
-            return t;
-        };
-        const float t = block_sum(l1_sum);
-        if (!l1_part) {
-            if (threadIdx.x == 0) atomicAdd(l1_loss, t * l1_inv_n);
-            return;
-        }
-        // the last block to get here adds up the blocks' parts (hundreds of them:
-        // an atomic sum would round each addition to the whole). The blocks are
-        // counted in the loss's own word, which is zero before this kernel
-        if (threadIdx.x == 0) {
-            __stcg(l1_part + blockIdx.x, t);
-            __threadfence();
-            s_item = atomicAdd(reinterpret_cast<unsigned int *>(l1_loss), 1u) == gridDim.x - 1;
-        }
+        for (int o = 16; o > 0; o >>= 1) l1_sum += __shfl_xor_sync(0xffffffffu, l1_sum, o);
+        if (lane == 0) s_l1[threadIdx.x >> 5] = l1_sum;
         __syncthreads();
-        if (!s_item) return;
-        __threadfence();
-        float sum = 0.f;
-#pragma unroll 8
-        for (int i = threadIdx.x; i < (int)gridDim.x; i += BS) sum += __ldcg(l1_part + i);
-        sum = block_sum(sum);
-        if (threadIdx.x == 0) *l1_loss = sum * l1_inv_n;
+        if (threadIdx.x == 0) {
+            float t = 0.f;
+            for (int w = 0; w < R::WARPS; ++w) t += s_l1[w];
+            add_loss(l1_loss, t * l1_inv_n, l1_carry);
+        }
     }
 }
 
-// Zero the raster backward's accumulators (the 2D gradients, and the L1 loss
-// when given) as a programmatic dependent of the kernel ahead on the stream
-// (in a step, the raster forward): nothing here touches what that kernel
+// Zero the raster backward's accumulators (the 2D gradients, and the L1 loss and its
+// carry when given), early as a programmatic dependent of the kernel ahead on the
+// stream (in a step, the raster forward): nothing here touches what that kernel
 // reads or writes, so the stores run on the SMs it leaves in its tail; the
 // wait at the end keeps the stream's order for the kernels after this one.
 __global__ void __launch_bounds__(256) k_zero_accumulators(float4 *__restrict__ p, long long n4,
-                                                           float *__restrict__ loss) {
+                                                           float *__restrict__ loss, float *__restrict__ carry) {
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n4; i += (long long)gridDim.x * 256) p[i] = z;
-    if (loss && blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.f;
+    if (loss && blockIdx.x == 0 && threadIdx.x == 0) *loss = *carry = 0.f;
     grid_dependency_wait();
 }
 
-int launch_zero_accumulators(float *grad2d, long long n_floats, float *loss, cudaStream_t st) {
+int launch_zero_accumulators(float *grad2d, long long n_floats, const L1Loss &l1, bool early, cudaStream_t st) {
     // (n_floats: 12 per slot, a whole number of float4; grad2d 16-byte aligned)
     const long long n4 = n_floats / 4;
     cudaLaunchConfig_t lc = {};
@@ -729,8 +728,9 @@ int launch_zero_accumulators(float *grad2d, long long n_floats, float *loss, cud
     lc.blockDim = dim3(256);
     lc.stream = st;
     lc.attrs = at;
-    lc.numAttrs = 1;
-    if (cudaLaunchKernelEx(&lc, k_zero_accumulators, reinterpret_cast<float4 *>(grad2d), n4, loss) != cudaSuccess)
+    lc.numAttrs = early ? 1 : 0;
+    if (cudaLaunchKernelEx(&lc, k_zero_accumulators, reinterpret_cast<float4 *>(grad2d), n4, l1.loss, l1.carry) !=
+        cudaSuccess)
         return GS_ERR_CUDA;
     return GS_OK;
 }
@@ -888,20 +888,11 @@ static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, co
     } else if (grid < items && cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, sizeof(int), st) != cudaSuccess) {
         return GS_ERR_CUDA;
     }
-    // the blocks' parts of the loss lie behind the work record (tile_scratch is
-    // 5 ints per tile, the grid at most one block per region). Two blocks per SM or
-    // more: their ordered sum has an error of 1e-7 where the atomic additions, each
-    // rounded to the whole, reach 1e-6, and costs a step 1 to 2 us (304 tiles of 16x16
-    // 84.4 -> 86.2 us, 2,170 of them 450 -> 452; 2,500 tiles of 8x8 173 -> 178). Fewer
-    // blocks add to the loss with atomics.
-    static_assert(R::PARTS <= 4, "one part of the loss per block fits tile_scratch");
-    const bool many = grid >= 2 * num_sms();
-    float *l1_part = l1.loss && b->tile_scratch && many
-                         ? reinterpret_cast<float *>(b->tile_scratch + L.n_tiles) : nullptr;
+    // (few blocks add to the loss without a carry: their error is 4e-7 at most)
     k_render_bwd<TW, TH, COUNT, LAST><<<grid, R::BS, smem, st>>>(
         L, reinterpret_cast<const float4 *>(proj), reinterpret_cast<const int2 *>(b->tile_ranges), b->ids,
         b->tile_order, b->counters, image, dL_dimage, b->last_contrib, reinterpret_cast<float4 *>(grad2d), l1.target,
-        l1.loss, l1.inv_n, l1_part);
+        l1.loss, l1.inv_n, grid >= 2 * num_sms() ? l1.carry : nullptr);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
