@@ -205,11 +205,11 @@ __device__ __forceinline__ void count_pairs(int *counters, int at, unsigned int 
 
 // One staged Gaussian: its three float4 lie together (48 bytes apart, an odd
 // number of 16-byte bank groups: no conflicts on the stores), so that a visit
-// reads them at one address.
+// reads them at one address. (s_ad: the backward's natural-log terms of the conic.)
 template <typename R>
 __device__ __forceinline__ void stage_one(const Launch &L, const float4 *__restrict__ proj,
                                           const unsigned int *__restrict__ ids, int index, int k, const TileInfo &ti,
-                                          float4 *s_st, typename R::Mask *s_mask, float2 *s_ad) {
+                                          float4 *s_st, typename R::Mask *s_mask, float2 *s_ad = nullptr) {
     float4 xy, con, rgb;
     stage(proj, ids[index], index, ti.ox, ti.oy, xy, con, rgb);
     s_st[3 * k] = xy;
@@ -219,7 +219,7 @@ __device__ __forceinline__ void stage_one(const Launch &L, const float4 *__restr
     s_mask[k] = (typename R::Mask)warp_mask<R::RW, R::RH>(xy, con, L.alpha_min, ti.tbx, ti.tby);
 }
 
-// Stage the next batch of a tile's instances [pos, end) that reach the block's
+// Stage the forward's next batch of a tile's instances [pos, end) that reach the block's
 // region: at most per BS of them (per: 1, 2 or 4 per thread, the batch size
 // chosen at launch), in list order; pos moves past the last one looked at.
 // Returns their number. With one part per tile every instance is taken (the
@@ -235,13 +235,12 @@ struct Pack {
 template <typename R>
 __device__ __forceinline__ int stage_batch(const Launch &L, const float4 *__restrict__ proj,
                                            const unsigned int *__restrict__ ids, int &pos, int end, int per,
-                                           const TileInfo &ti, float4 *s_st, typename R::Mask *s_mask, Pack *pk,
-                                           float2 *s_ad = nullptr) {
+                                           const TileInfo &ti, float4 *s_st, typename R::Mask *s_mask, Pack *pk) {
     constexpr int BS = R::BS;
     if constexpr (R::PARTS == 1) {
         for (int h = 0; h < per; ++h) {
             const int k = threadIdx.x + h * BS;
-            if (k < end - pos) stage_one<R>(L, proj, ids, pos + k, k, ti, s_st, s_mask, s_ad);
+            if (k < end - pos) stage_one<R>(L, proj, ids, pos + k, k, ti, s_st, s_mask);
         }
         const int nb = min(per * BS, end - pos);
         pos += nb;
@@ -283,7 +282,7 @@ __device__ __forceinline__ int stage_batch(const Launch &L, const float4 *__rest
             const int k = base + __popc(bal & ((1u << lane) - 1u));
             const int i = pos + j * BS + threadIdx.x;
             if (bal >> lane & 1u) {
-                if (k < cap) stage_one<R>(L, proj, ids, i, k, ti, s_st, s_mask, s_ad);
+                if (k < cap) stage_one<R>(L, proj, ids, i, k, ti, s_st, s_mask);
                 else if (k == cap) pk->next = i;   // the first that did not fit starts the next batch
             }
         }
@@ -431,6 +430,10 @@ __global__ void __launch_bounds__(FwdRegion<TW, TH>::BS, 1024 / FwdRegion<TW, TH
 // last composited one), so every Gaussian that passes the alpha test there
 // is composited, and the warp and the block stop at their pixels' largest
 // end instead of walking on to saturation or the end of the list.
+// The kernel sits at its 64-register cap, and what lives across its loops shows in
+// all of it: the next item formed in a register (as in the forward) cost 10 us of 320,
+// staging through the forward's function, with its position in the list, 8 (1M view,
+// 32x32 tiles). So the next item waits in shared memory and the staging is written out.
 // Add a block's part to the loss. Every addition rounds to the whole: hundreds of
 // them leave an error of 1e-6. With a carry word (zero before the kernel) what an
 // addition rounds away, which the old value and the part give exactly, goes there,
@@ -465,6 +468,7 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
     // the conic's A and D (natural-log units), the per-Gaussian gradient sums
     // (pitch 9, odd: no bank conflicts) and warp masks
     using R = BwdRegion<TW, TH>;
+    static_assert(R::PARTS == 1, "a block per tile");
     constexpr int BS = R::BS;
     const int NB = L.bwd_batch * BS;
     extern __shared__ float4 s_dyn[];
@@ -474,7 +478,6 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
     float *s_g = reinterpret_cast<float *>(s_ad + NB);
     typename R::Mask *s_mask = reinterpret_cast<typename R::Mask *>(s_g + 9 * NB);
     __shared__ int s_item;
-    __shared__ Pack s_pack;
     __shared__ float s_l1[R::WARPS];
     // the projection backward that follows (launched as a programmatic
     // dependent) may start its blocks on SMs this kernel leaves in its tail:
@@ -492,11 +495,14 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
     const float4 *red_row = reinterpret_cast<const float4 *>(rb + lane * RED_PITCH);
     for (int k = threadIdx.x; k < 9 * NB; k += BS) s_g[k] = 0.f;
     float l1_sum = 0.f;   // with l1_target: this thread's sum of |image - target|
-    const int items = L.n_tiles * R::PARTS;
-    __syncthreads();   // the sums are zero
-    for (int item = blockIdx.x; item < items; item = next_item(counters + CNT_Q_BWD, items, &s_item)) {
-        const int tile = order[item / R::PARTS];
-        const TileInfo ti = tile_info<R>(L, tile, item % R::PARTS);
+    if (threadIdx.x == 0) s_item = blockIdx.x;
+    for (;;) {
+        __syncthreads();   // (at first also: the sums are zero)
+        const int item = s_item;
+        __syncthreads();
+        if (item >= L.n_tiles) break;
+        const int tile = order[item];
+        const TileInfo ti = tile_info<R>(L, tile, 0);
         const int2 r = ranges[tile];
         const ViewDesc &vd = L.v[ti.view];
         const long long hw = (long long)vd.W * vd.H;
@@ -565,12 +571,17 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
             npend = 0;
             __syncwarp();   // the buffer is free for the next visits
         };
-        for (int pos = r.x; pos < r.y;) {
-            if (__syncthreads_count(LAST ? pos >= endm : done0 && done1) == BS) break;
-            const int nb = stage_batch<R>(L, proj, ids, pos, r.y, L.bwd_batch, ti, s_st, s_mask, &s_pack, s_ad);
+        for (int b0 = r.x, nb; b0 < r.y; b0 += nb) {
+            if (__syncthreads_count(LAST ? b0 >= endm : done0 && done1) == BS) break;
+            nb = min(NB, r.y - b0);
+            for (int h = 0; h < L.bwd_batch; ++h) {
+                const int k = threadIdx.x + h * BS;
+                if (k < nb) stage_one<R>(L, proj, ids, b0 + k, k, ti, s_st, s_mask, s_ad);
+            }
+            __syncthreads();
             for (int k0 = 0; k0 < nb; k0 += 32) {
                 // the warp's pixels have all stopped
-                if (__all_sync(0xffffffffu, LAST ? __float_as_int(s_st[3 * k0 + 2].w) >= endm : done0 && done1)) break;
+                if (__all_sync(0xffffffffu, LAST ? b0 + k0 >= endm : done0 && done1)) break;
                 // only the staged Gaussians that may reach this warp's patch, in order
                 unsigned int hits = __ballot_sync(0xffffffffu, k0 + lane < nb && (s_mask[k0 + lane] & wbit));
                 while (hits) {
@@ -689,6 +700,13 @@ __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH
             }
         }
         if (COUNT) count_pairs(counters, 12, n_eval, n_comp);
+        // The next tile. Every tile is followed by one fetch, so that the last of them
+        // leaves the queue at zero for the next call.
+        if (threadIdx.x == 0) {
+            const int fetch = atomicAdd(counters + CNT_Q_BWD, 1);
+            if (fetch == L.n_tiles - 1) counters[CNT_Q_BWD] = 0;
+            s_item = (int)gridDim.x + fetch;
+        }
     }
     if (l1_loss) {
         // the block's part of the loss
@@ -876,17 +894,14 @@ static int launch_bwd_c(const Launch &L, const float *proj, const gs_bins *b, co
     using R = BwdRegion<TW, TH>;
     static int blocks_per_sm[5];
     const size_t smem = (size_t)BWD_STAGE_BYTES<R> * L.bwd_batch * R::BS + sizeof(float) * RED_WARP_FLOATS * R::WARPS;
-    const long long items = (long long)L.n_tiles * R::PARTS;
-    const int grid = (int)min((long long)num_sms() * raster_blocks_per_sm(k_render_bwd<TW, TH, COUNT, LAST>, R::BS,
-                                                                          smem, L.bwd_batch, blocks_per_sm),
-                              max(1LL, items));
+    const int grid = min(num_sms() * raster_blocks_per_sm(k_render_bwd<TW, TH, COUNT, LAST>, R::BS, smem, L.bwd_batch,
+                                                          blocks_per_sm),
+                         max(1, (int)L.n_tiles));
     if (order_by_work(L, b) && !all_at_once<TW, TH>(L)) {
         // by the replay lengths that the forward recorded
         k_order_by_work<<<1, 1024, 0, st>>>(work_record(b), nullptr, (int)L.n_tiles, b->tile_order, false,
                                             b->counters + CNT_Q_BWD);
         if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-    } else if (grid < items && cudaMemsetAsync(b->counters + CNT_Q_BWD, 0, sizeof(int), st) != cudaSuccess) {
-        return GS_ERR_CUDA;
     }
     // (few blocks add to the loss without a carry: their error is 4e-7 at most)
     k_render_bwd<TW, TH, COUNT, LAST><<<grid, R::BS, smem, st>>>(
