@@ -139,7 +139,8 @@ typedef struct gs_bins {
     int32_t *tile_order;  /* [T] work order: tiles by decreasing instance count */
     int32_t *tile_scratch;/* [5T] scratch (per-tile counters, then the runs of large tiles that
                              are sorted in pieces) */
-    int32_t *counters;    /* [GS_NUM_COUNTERS] scratch; counters[0] = instances after the call;
+    int32_t *counters;    /* [GS_NUM_COUNTERS] scratch, prepared by gs_bin_sort (zero for lists built by
+                             hand) and kept between calls; counters[0] = instances after the call;
                              int64 at counters+8: pixel-Gaussian pairs evaluated by gs_render_fwd,
                              +10: composited by it, +12/+14: the same for gs_rasterize_bwd */
     int32_t *last_contrib;/* optional [sum_v H_v W_v] (NULL = not kept): per pixel (view v's pixel

@@ -424,16 +424,6 @@ __global__ void __launch_bounds__(FwdRegion<TW, TH>::BS, 1024 / FwdRegion<TW, TH
     }
 }
 
-// With LAST, each pixel's replay ends at the position after its last
-// composited Gaussian, which the forward recorded in last_contrib: no
-// Gaussian before that position stops the pixel (the stop comes after the
-// last composited one), so every Gaussian that passes the alpha test there
-// is composited, and the warp and the block stop at their pixels' largest
-// end instead of walking on to saturation or the end of the list.
-// The kernel sits at its 64-register cap, and what lives across its loops shows in
-// all of it: the next item formed in a register (as in the forward) cost 10 us of 320,
-// staging through the forward's function, with its position in the list, 8 (1M view,
-// 32x32 tiles). So the next item waits in shared memory and the staging is written out.
 // Add a block's part to the loss. Every addition rounds to the whole: hundreds of
 // them leave an error of 1e-6. With a carry word (zero before the kernel) what an
 // addition rounds away, which the old value and the part give exactly, goes there,
@@ -455,6 +445,16 @@ __device__ __forceinline__ void add_loss(float *loss, float part, float *carry) 
     if (more != 0.f) atomicAdd(carry, add(more));
 }
 
+// With LAST, each pixel's replay ends at the position after its last
+// composited Gaussian, which the forward recorded in last_contrib: no
+// Gaussian before that position stops the pixel (the stop comes after the
+// last composited one), so every Gaussian that passes the alpha test there
+// is composited, and the warp and the block stop at their pixels' largest
+// end instead of walking on to saturation or the end of the list.
+// The kernel sits at its 64-register cap, and what lives across its loops shows in
+// all of it: the next item formed in a register (as in the forward) cost 10 us of 320,
+// staging through the forward's function, with its position in the list, 8 (1M view,
+// 32x32 tiles). So the next item waits in shared memory and the staging is written out.
 template <int TW, int TH, bool COUNT, bool LAST>
 __global__ void __launch_bounds__(BwdRegion<TW, TH>::BS, 1024 / BwdRegion<TW, TH>::BS)
     k_render_bwd(const Launch L, const float4 *__restrict__ proj, const int2 *__restrict__ ranges,
